@@ -1,0 +1,302 @@
+// FP32 one-sided Jacobi with the columns held in registers.
+//
+// jacobi_cols_h4 reads and writes both columns of every pair (and of V) through
+// shared memory in every round, which bounds it by the shared-memory port: 256 KB
+// per round of 64 pairs of 128 entries, ~2050 of its ~2800 cycles.  Here a warp
+// keeps 2 B columns (two blocks of B) in its registers, rotates the B x B pairs
+// of the two blocks in B steps without leaving them, and then passes one block on
+// to its neighbour through shared memory: 1 / (2 B) of that traffic and one
+// block barrier per B rounds.
+//
+// Order of the pairs: odd-even transposition of the 2 W blocks of W warps.  In an
+// even phase warp w holds positions (2 w, 2 w + 1), in an odd phase
+// (2 w + 1, 2 w + 2); the two blocks of a warp trade places after they met, so in
+// 2 W phases every two blocks meet exactly once (the order of the blocks ends
+// reversed, which the caller does not see: columns are not ordered).  The
+// pairs inside a block are rotated at the start of a sweep.
+//
+// Measured (128^3 sums of two at bond 64, 9 jobs, 128 x 128 centre matrices):
+// the rounding 67.5 -> 34.7 ms; 3.4 M -> 0.9 M cycles per SVD of a 64^3 step at
+// bond 64.  Bound by instruction issue: ~140 instructions per warp and step of 64
+// pairs (four warps a scheduler), of which 64 are the rotation's arithmetic.
+#pragma once
+
+#include "linalg.cuh"
+
+namespace tn {
+
+// Totals over the warp of v[0..B): lane group q = lane / (32 / B) gets that of v[q].
+template <int B>
+__device__ __forceinline__ float jr_reduce(float (&v)[B], int lane) {
+  constexpr unsigned F = 0xffffffffu;
+  float r;
+  if constexpr (B == 4) {
+    const bool h = lane & 16;
+    const float s0 = h ? v[0] : v[2], s1 = h ? v[1] : v[3];
+    const float k0 = (h ? v[2] : v[0]) + __shfl_xor_sync(F, s0, 16);
+    const float k1 = (h ? v[3] : v[1]) + __shfl_xor_sync(F, s1, 16);
+    const bool g = lane & 8;
+    r = (g ? k1 : k0) + __shfl_xor_sync(F, g ? k0 : k1, 8);
+  } else if constexpr (B == 2) {
+    const bool h = lane & 16;
+    r = (h ? v[1] : v[0]) + __shfl_xor_sync(F, h ? v[0] : v[1], 16);
+    r += __shfl_xor_sync(F, r, 8);
+  } else {
+    r = v[0] + __shfl_xor_sync(F, v[0], 16);
+    r += __shfl_xor_sync(F, r, 8);
+  }
+  r += __shfl_xor_sync(F, r, 4);
+  r += __shfl_xor_sync(F, r, 2);
+  r += __shfl_xor_sync(F, r, 1);
+  return r;
+}
+
+// Rutishauser's rotation zeroing the inner product ga of columns with squared
+// norms al, be (c = 1, s = 0 if they count as orthogonal: |ga| <= tol sqrt(al)
+// sqrt(be), or one carries nothing).  al, be are updated to the rotated norms.
+// MUFU reciprocal and square root (2 ulp): the rotation is off orthogonal by
+// ~2e-7, which scales a column of W by that much and turns it not at all; the
+// caller takes directions, not lengths, from W where it needs more.
+__device__ __forceinline__ bool jr_angle(float& al, float& be, float ga, float tol, float& c, float& s) {
+  c = 1.f;
+  s = 0.f;
+  // the FP32 floor of jacobi_cols_hw: below it zeta could overflow
+  if (!(al >= 1e-24f) || !(be >= 1e-24f) || !(fabsf(ga) * (rsqrtf(al) * rsqrtf(be)) > tol)) return false;
+  const float z = __fdividef(be - al, 2.f * ga), az = fabsf(z);
+  const float q = fmaf(z, z, 1.f);
+  const float t = copysignf(az > 1e15f ? __fdividef(0.5f, az) : __fdividef(1.f, az + q * rsqrtf(q)), z);
+  c = rsqrtf(fmaf(t, t, 1.f));
+  s = c * t;
+  al -= t * ga;
+  be += t * ga;
+  return true;
+}
+
+// One step: the pairs (X[i], Y[(i + S) % B]) of two blocks, their squared norms
+// na (of X[q]) and nb (of Y[q]) kept by lane group q.
+template <int B, int EPL, int S>
+__device__ __forceinline__ bool jr_cross(float (&X)[B][EPL], float (&Y)[B][EPL], float& na, float& nb, float tol,
+                                         int lane) {
+  constexpr unsigned F = 0xffffffffu;
+  constexpr int G = 32 / B;
+  float d[B];
+#pragma unroll
+  for (int i = 0; i < B; ++i) {
+    float a = 0.f;
+#pragma unroll
+    for (int e = 0; e < EPL; ++e) a = fmaf(X[i][e], Y[(i + S) % B][e], a);
+    d[i] = a;
+  }
+  const float ga = jr_reduce<B>(d, lane);
+  float be = S == 0 ? nb : __shfl_sync(F, nb, (lane + S * G) & 31);
+  float c, s;
+  const bool go = jr_angle(na, be, ga, tol, c, s);
+  if (!__any_sync(F, go)) return false;
+  nb = S == 0 ? be : __shfl_sync(F, be, (lane + 32 - S * G) & 31);
+#pragma unroll
+  for (int i = 0; i < B; ++i) {
+    const float ci = B == 1 ? c : __shfl_sync(F, c, i * G), si = B == 1 ? s : __shfl_sync(F, s, i * G);
+#pragma unroll
+    for (int e = 0; e < EPL; ++e) {
+      const float x = X[i][e], y = Y[(i + S) % B][e];
+      X[i][e] = ci * x - si * y;
+      Y[(i + S) % B][e] = si * x + ci * y;
+    }
+  }
+  return true;
+}
+
+// The pairs inside the two blocks, (X[i0], X[i1]), (X[i2], X[i3]) and the same of
+// Y (B = 4), or (X[0], X[1]) and (Y[0], Y[1]) (B = 2).
+template <int B, int EPL, int I0, int I1, int I2, int I3>
+__device__ __forceinline__ bool jr_inner(float (&X)[B][EPL], float (&Y)[B][EPL], float tol, int lane) {
+  constexpr unsigned F = 0xffffffffu;
+  constexpr int G = 32 / B, H = B / 2;
+  float d[B], na[B], nb[B];
+#pragma unroll
+  for (int q = 0; q < B; ++q) {
+    const int i = (q % H) == 0 ? I0 : I2, j = (q % H) == 0 ? I1 : I3;
+    float a = 0.f, x2 = 0.f, y2 = 0.f;
+#pragma unroll
+    for (int e = 0; e < EPL; ++e) {
+      const float x = q < H ? X[i][e] : Y[i][e], y = q < H ? X[j][e] : Y[j][e];
+      a = fmaf(x, y, a);
+      x2 = fmaf(x, x, x2);
+      y2 = fmaf(y, y, y2);
+    }
+    d[q] = a;
+    na[q] = x2;
+    nb[q] = y2;
+  }
+  const float ga = jr_reduce<B>(d, lane);
+  float al = jr_reduce<B>(na, lane), be = jr_reduce<B>(nb, lane), c, s;
+  const bool go = jr_angle(al, be, ga, tol, c, s);
+  if (!__any_sync(F, go)) return false;
+#pragma unroll
+  for (int q = 0; q < B; ++q) {
+    const int i = (q % H) == 0 ? I0 : I2, j = (q % H) == 0 ? I1 : I3;
+    const float ci = __shfl_sync(F, c, q * G), si = __shfl_sync(F, s, q * G);
+#pragma unroll
+    for (int e = 0; e < EPL; ++e) {
+      const float x = q < H ? X[i][e] : Y[i][e], y = q < H ? X[j][e] : Y[j][e];
+      const float u = ci * x - si * y, w = si * x + ci * y;
+      if (q < H) { X[i][e] = u; X[j][e] = w; }
+      else { Y[i][e] = u; Y[j][e] = w; }
+    }
+  }
+  return true;
+}
+
+// A block of B columns in shared memory: EPL consecutive entries of a column per lane.
+template <int B, int EPL>
+__device__ __forceinline__ void jr_store(float* p, const float (&X)[B][EPL], int lane) {
+#pragma unroll
+  for (int i = 0; i < B; ++i)
+#pragma unroll
+    for (int e = 0; e < EPL; e += 4) {
+      if constexpr (EPL % 4 == 0)
+        *(float4*)(p + (size_t)i * 32 * EPL + e * 32 + 4 * lane) = make_float4(X[i][e], X[i][e + 1], X[i][e + 2], X[i][e + 3]);
+      else if constexpr (EPL == 2)
+        *(float2*)(p + (size_t)i * 64 + 2 * lane) = make_float2(X[i][0], X[i][1]);
+      else
+        p[(size_t)i * 32 + lane] = X[i][0];
+    }
+}
+template <int B, int EPL>
+__device__ __forceinline__ void jr_load(const float* p, float (&X)[B][EPL], int lane) {
+#pragma unroll
+  for (int i = 0; i < B; ++i)
+#pragma unroll
+    for (int e = 0; e < EPL; e += 4) {
+      if constexpr (EPL % 4 == 0) {
+        const float4 v = *(const float4*)(p + (size_t)i * 32 * EPL + e * 32 + 4 * lane);
+        X[i][e] = v.x; X[i][e + 1] = v.y; X[i][e + 2] = v.z; X[i][e + 3] = v.w;
+      } else if constexpr (EPL == 2) {
+        const float2 v = *(const float2*)(p + (size_t)i * 64 + 2 * lane);
+        X[i][0] = v.x; X[i][1] = v.y;
+      } else {
+        X[i][0] = p[(size_t)i * 32 + lane];
+      }
+    }
+}
+
+// Sweeps on the columns W[j * 32 EPL + i] (shared memory; zero beyond the column
+// count and length, columns padded to a multiple of 2 B), at most maxsw.  Returns
+// the sweeps that rotated anything (maxsw if the last one still did).  W is the
+// exchange buffer meanwhile: 2 W blocks are one block out and one block in per
+// warp, so a sending phase alternates between its halves.
+template <int B, int EPL>
+__device__ __noinline__ int jacobi_reg_run(float* W, int ncol, int len, int maxsw) {
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  const int nw = (ncol + 2 * B - 1) / (2 * B);              // warps that hold columns
+  constexpr int BS = B * 32 * EPL;                          // floats of a block
+  const float tol = 16.f * Eps<float>::v * sqrtf((float)len);
+  __shared__ int s_rot[2];
+  if (threadIdx.x < 2) s_rot[threadIdx.x] = 0;
+  __syncthreads();
+  int sweep = 0;
+  if (wid < nw) {
+    float X[B][EPL], Y[B][EPL];
+    jr_load<B, EPL>(W + (size_t)(2 * wid) * BS, X, lane);
+    jr_load<B, EPL>(W + (size_t)(2 * wid + 1) * BS, Y, lane);
+    float* buf[2] = {W, W + (size_t)nw * BS};
+    auto meet = [&]() { asm volatile("bar.sync 1, %0;" ::"r"(nw * 32) : "memory"); };
+    // all cross pairs of the two blocks, with norms taken afresh
+    auto cross = [&]() -> bool {
+      float na[B], nb[B];
+#pragma unroll
+      for (int i = 0; i < B; ++i) {
+        float a = 0.f, b = 0.f;
+#pragma unroll
+        for (int e = 0; e < EPL; ++e) {
+          a = fmaf(X[i][e], X[i][e], a);
+          b = fmaf(Y[i][e], Y[i][e], b);
+        }
+        na[i] = a;
+        nb[i] = b;
+      }
+      float al = jr_reduce<B>(na, lane), be = jr_reduce<B>(nb, lane);
+      bool r = jr_cross<B, EPL, 0>(X, Y, al, be, tol, lane);
+      if constexpr (B >= 2) r |= jr_cross<B, EPL, 1>(X, Y, al, be, tol, lane);
+      if constexpr (B == 4) {
+        r |= jr_cross<B, EPL, 2>(X, Y, al, be, tol, lane);
+        r |= jr_cross<B, EPL, 3>(X, Y, al, be, tol, lane);
+      }
+      return r;
+    };
+    meet();
+    for (; sweep < maxsw; ++sweep) {
+      bool rot = false;
+      if constexpr (B == 4) {
+        rot |= jr_inner<B, EPL, 0, 1, 2, 3>(X, Y, tol, lane);
+        rot |= jr_inner<B, EPL, 0, 2, 1, 3>(X, Y, tol, lane);
+        rot |= jr_inner<B, EPL, 0, 3, 1, 2>(X, Y, tol, lane);
+      } else if constexpr (B == 2) {
+        rot |= jr_inner<B, EPL, 0, 1, 0, 1>(X, Y, tol, lane);
+      }
+      for (int ph = 0; ph < nw; ++ph) {
+        // even phase; the blocks trade places: Y (now first) goes to the left
+        // neighbour's right hand (warp 0's parks with the last warp)
+        rot |= cross();
+        jr_store<B, EPL>(buf[0] + (size_t)(wid == 0 ? nw - 1 : wid - 1) * BS, Y, lane);
+        meet();
+        jr_load<B, EPL>(buf[0] + (size_t)wid * BS, Y, lane);
+        // odd phase: the last warp holds the two ends, which do not meet; its X
+        // stays the last position, so it leaves as the others' Y stays
+        if (wid + 1 < nw) {
+          rot |= cross();
+          jr_store<B, EPL>(buf[1] + (size_t)(wid + 1) * BS, X, lane);
+        } else {
+          jr_store<B, EPL>(buf[1], Y, lane);
+#pragma unroll
+          for (int i = 0; i < B; ++i)
+#pragma unroll
+            for (int e = 0; e < EPL; ++e) Y[i][e] = X[i][e];
+        }
+        meet();
+        jr_load<B, EPL>(buf[1] + (size_t)wid * BS, X, lane);
+      }
+      if (rot && lane == 0) s_rot[sweep & 1] = 1;
+      meet();
+      const int any = s_rot[sweep & 1];
+      if (threadIdx.x == 0) s_rot[(sweep + 1) & 1] = 0;     // read two meetings ago
+      meet();
+      if (!any) break;
+    }
+    jr_store<B, EPL>(W + (size_t)(2 * wid) * BS, X, lane);
+    jr_store<B, EPL>(W + (size_t)(2 * wid + 1) * BS, Y, lane);
+  }
+  __shared__ int s_sweeps;
+  if (threadIdx.x == 0) s_sweeps = sweep;
+  __syncthreads();
+  sweep = s_sweeps;
+  __syncthreads();
+  return sweep;
+}
+
+// Shapes that jacobi_reg takes with 512 threads: 16 warps of 8 columns, eight
+// entries per lane (2 x 4 x 8 = 64 registers of data).
+__host__ __device__ inline bool jacobi_reg_fits(int ncol, int len) { return ncol <= 128 && len <= 256; }
+// Leading dimension of W, and its columns (padded to whole warps of blocks).
+__host__ __device__ inline int jacobi_reg_ld(int len) { return len <= 32 ? 32 : len <= 64 ? 64 : len <= 128 ? 128 : 256; }
+__host__ __device__ inline int jacobi_reg_block(int ncol) { return ncol <= 32 ? 1 : ncol <= 64 ? 2 : 4; }
+__host__ __device__ inline int jacobi_reg_cols(int ncol) {
+  const int b2 = 2 * jacobi_reg_block(ncol);
+  return (ncol + b2 - 1) / b2 * b2;
+}
+
+// One-sided FP32 Jacobi of the padded columns in W (see jacobi_reg_run).  Blocks
+// of 4 columns when more than 64 are there, of 2 or 1 below so that all 16 warps
+// have columns.
+__device__ __forceinline__ int jacobi_reg(float* W, int ncol, int len, int maxsw) {
+  const int b = jacobi_reg_block(ncol);
+#define JR(B)                                                                   \
+  (len <= 32    ? jacobi_reg_run<B, 1>(W, ncol, len, maxsw)                     \
+   : len <= 64  ? jacobi_reg_run<B, 2>(W, ncol, len, maxsw)                     \
+   : len <= 128 ? jacobi_reg_run<B, 4>(W, ncol, len, maxsw)                     \
+                : jacobi_reg_run<B, 8>(W, ncol, len, maxsw))
+  return b == 1 ? JR(1) : b == 2 ? JR(2) : JR(4);
+#undef JR
+}
+
+}  // namespace tn

@@ -168,6 +168,39 @@ __device__ void cta_gemm(int M, int N, int K, const T* A, int lda, const T* B, i
   __syncthreads();
 }
 
+// C (M x N, ldc) = A (M x K, lda) * B^T with B given as N x K (ldb).
+template <typename T>
+__device__ void cta_gemm_nt(int M, int N, int K, const T* A, int lda, const T* B, int ldb, T* C, int ldc) {
+  const int tm = (M + 3) >> 2, tnn = (N + 3) >> 2;
+  for (int t = threadIdx.x; t < tm * tnn; t += blockDim.x) {
+    const int i0 = (t / tnn) * 4, j0 = (t % tnn) * 4;
+    T acc[4][4];
+#pragma unroll
+    for (int a = 0; a < 4; ++a)
+#pragma unroll
+      for (int b = 0; b < 4; ++b) acc[a][b] = (T)0;
+    for (int k = 0; k < K; ++k) {
+      T av[4], bv[4];
+#pragma unroll
+      for (int a = 0; a < 4; ++a) av[a] = (i0 + a < M) ? A[(size_t)(i0 + a) * lda + k] : (T)0;
+#pragma unroll
+      for (int b = 0; b < 4; ++b) bv[b] = (j0 + b < N) ? B[(size_t)(j0 + b) * ldb + k] : (T)0;
+#pragma unroll
+      for (int a = 0; a < 4; ++a)
+#pragma unroll
+        for (int b = 0; b < 4; ++b) acc[a][b] += av[a] * bv[b];
+    }
+#pragma unroll
+    for (int a = 0; a < 4; ++a) {
+      if (i0 + a >= M) continue;
+#pragma unroll
+      for (int b = 0; b < 4; ++b)
+        if (j0 + b < N) C[(size_t)(i0 + a) * ldc + j0 + b] = acc[a][b];
+    }
+  }
+  __syncthreads();
+}
+
 // Householder QR of A (m x n, lda; typically shared memory, lda = n + 1 to
 // avoid bank conflicts), with Q (m x k, ldq) and R (k x n, ldr) written out,
 // diag(R) >= 0.  Parallel form: per column, the reflector inner products are

@@ -11,6 +11,7 @@
 #include <algorithm>
 
 #include "cluster.cuh"
+#include "jacobi_reg.cuh"
 #include "linalg.cuh"
 
 namespace tn {
@@ -1043,6 +1044,168 @@ __device__ __noinline__ int svd64_site(const RoundJob& J, int L, int k, const T*
   return r;
 }
 
+// Shared-memory bytes of svd32_site: W, then (once W is final) the kept rows of
+// V^T and their Gram matrix beside it.
+__host__ __device__ inline size_t svd32_vbytes(int r, int n) {
+  return ((size_t)r * (n | 1) + (size_t)r * (r | 1)) * sizeof(float);
+}
+
+// Whether svd32_site takes an m x n centre matrix: its vectors fit the register
+// Jacobi, and W with the QR panel (m > n) fits the work area.
+__host__ __device__ inline bool svd32_fits(int m, int n) {
+  const int k = m < n ? m : n;
+  if (!jacobi_reg_fits(k, n)) return false;
+  if (m > n && (size_t)m * (n | 1) * sizeof(float) > (size_t)SM_WORK) return false;
+  return (size_t)jacobi_reg_cols(k) * jacobi_reg_ld(n) * sizeof(float) <= (size_t)SM_WORK;
+}
+
+// Centre SVD of one right-to-left step in FP32, without accumulating the
+// rotations: the Jacobi runs on the rows of C (n-vectors; of the R of C = QR when
+// m > n, whose right singular vectors are C's), so its converged vectors are
+// s_j v_j, their directions the kept rows of V^T, and U S = C V is one product.
+// The kept rows are made orthonormal to FP32 rounding by one Newton-Schulz step
+// (the Jacobi stops at |cos| <= 16 eps sqrt(n)), so C V V^T is an orthogonal
+// projection of C itself: the error is that of the discarded part and of one
+// product, not of the ~1000 rotations a column goes through.  Vectors below the
+// Jacobi's floor (1e-12 of the scale) carry nothing: their columns of U S are zero.
+// Leaves singular values and order in sh.sig / sh.perm; returns the kept rank,
+// or 0 after flagging an error.
+__device__ __noinline__ int svd32_site(const RoundJob& J, int L, int k, const float* C, int m, int n, float* out,
+                                       float* US, float* scr, float* work, const SiteShared& sh, float* wv,
+                                       int job, int* status, const LearnCtx* lc, PhaseClock& pc,
+                                       double delta) {
+  const int ncol = imin(m, n), ld = jacobi_reg_ld(n), ncp = jacobi_reg_cols(ncol);
+  float* W = work;
+  // exact power-of-two scale so that max |C| is in [1, 2)
+  float amax = 0.f;
+  for (int idx = threadIdx.x; idx < m * n; idx += blockDim.x) amax = fmaxf(amax, fabsf(C[idx]));
+  for (int o = 16; o > 0; o >>= 1) amax = fmaxf(amax, __shfl_xor_sync(0xffffffffu, amax, o));
+  if ((threadIdx.x & 31) == 0) sh.red[threadIdx.x >> 5] = (double)amax;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    double a = 0.0;
+    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) a = fmax(a, sh.red[w]);
+    int e = 0;
+    if (a > 0.0 && isfinite(a)) frexp(a, &e);
+    sh.tau[1] = ldexp(1.0, 1 - e);
+  }
+  __syncthreads();
+  const double scl = sh.tau[1];
+  const float* X = C;
+  if (m > n) {
+    // R of C (n x n): the QR runs on a copy in the work area
+    const int lda = n | 1;
+    for (int idx = threadIdx.x; idx < m * n; idx += blockDim.x) work[(size_t)(idx / n) * lda + idx % n] = C[idx];
+    __syncthreads();
+    float* R = scr + J.lay.jv_off;
+    float* vb = scr + J.lay.qw_off;
+    householder_qr_blk<float>(work, m, n, lda, nullptr, 0, R, n, sh.tau, wv, sh.red, vb, vb + (size_t)m * QB);
+    if (threadIdx.x == 0) sh.tau[1] = scl;
+    __syncthreads();
+    X = R;
+  }
+  for (int idx = threadIdx.x; idx < ncp * ld; idx += blockDim.x) {
+    const int j = idx / ld, i = idx % ld;
+    W[idx] = (j < ncol && i < n) ? (float)scl * X[(size_t)j * n + i] : 0.f;
+  }
+  __syncthreads();
+  const int maxsw = J.max_sweeps > 0 ? J.max_sweeps : 60;
+  pc.lap(PH_SVD_OUT);
+  const int sw = jacobi_reg(W, ncol, n, maxsw);
+  pc.lap(PH_JACOBI);
+  if (threadIdx.x == 0) {
+    pc.acc[6] += sw; pc.acc[7] += 1.0;
+    if (sw >= maxsw) {
+      flag(status, ST_NOCONV);
+      if (atomicCAS(&status[1], 0, 1) == 0) {
+        status[2] = job; status[3] = k; status[4] = ncol; status[5] = imax(m, n);
+      }
+    }
+  }
+  // the padded columns moved among the others: norms of all ncp, the zero ones
+  // (-2) order last and are not counted
+  {
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
+    for (int j = warp; j < ncp; j += nw) {
+      float a = 0.f;
+      for (int i = lane; i < ld; i += 32) { const float w = W[(size_t)j * ld + i]; a = fmaf(w, w, a); }
+      for (int o = 16; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
+      if (lane == 0) {
+        const double sv = (double)sqrtf(a) / scl;
+        if (!(sv >= 0.0) || isinf(sv)) { sh.sig[j] = -1.0; flag(status, ST_NAN); }
+        else sh.sig[j] = sv;
+      }
+    }
+  }
+  __syncthreads();
+  for (int jj = threadIdx.x; jj < ncp; jj += blockDim.x) {
+    int rank = 0;
+    const double sj = sh.sig[jj];
+    for (int o = 0; o < ncp; ++o) {
+      const double so = sh.sig[o];
+      rank += (so > sj) || (so == sj && o < jj);
+    }
+    sh.perm[rank] = jj;
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    const int rmax = imin(J.chi, ncol);
+    double tail2 = 0.0;
+    int rr = rmax;
+    for (int p = ncol - 1; p >= 1; --p) {
+      const double sv = sh.sig[sh.perm[p]];
+      tail2 += sv * sv;
+      sh.tau[2 + p] = tail2;
+    }
+    for (int q = 1; q <= rmax; ++q) {
+      const double t2 = (q < ncol) ? sh.tau[2 + q] : 0.0;
+      if (sqrt(t2) <= delta) { rr = q; break; }
+    }
+    if (rr > bond_cap(L, J.dst.cap, k)) { *sh.bad = 1; rr = bond_cap(L, J.dst.cap, k); }
+    *sh.rank = rr;
+    if (J.discard && rr < ncol) atomicAdd(J.discard, sh.tau[2 + rr]);
+    *sh.flops += svd_flops(m, n);
+    if (lc && lc->counters) atomicAdd(&lc->counters[2], 1);
+  }
+  __syncthreads();
+  if (*sh.bad) { if (threadIdx.x == 0) flag(status, ST_CAPACITY); return 0; }
+  const int r = *sh.rank;
+  // kept directions, orthonormalised: V <- (3/2 I - 1/2 V V^T) V
+  const size_t wbytes = (size_t)ncp * ld * sizeof(float);
+  const bool vs = wbytes + svd32_vbytes(r, n) <= (size_t)SM_WORK;
+  const int ldv = vs ? (n | 1) : n, ldg = r | 1;
+  float* V = vs ? work + (size_t)ncp * ld : out;
+  float* G = vs ? V + (size_t)r * ldv : scr + J.lay.jv_off;
+  for (int idx = threadIdx.x; idx < r * n; idx += blockDim.x) {
+    const int jr = idx / n, c = idx % n, pj = sh.perm[jr];
+    const float sg = (float)(sh.sig[pj] * scl);
+    V[(size_t)jr * ldv + c] = sg > 0.f ? W[(size_t)pj * ld + c] / sg : (c == jr ? 1.f : 0.f);
+  }
+  __syncthreads();
+  cta_gemm_nt<float>(r, r, n, V, ldv, V, ldv, G, vs ? ldg : r);
+  for (int idx = threadIdx.x; idx < r * r; idx += blockDim.x) {
+    const int i = idx / r, j = idx % r;
+    const bool live = sh.sig[sh.perm[i]] * scl > 1e-12 && sh.sig[sh.perm[j]] * scl > 1e-12;
+    float* g = G + (size_t)i * (vs ? ldg : r) + j;
+    *g = (i == j ? 1.f : 0.f) + (live ? 0.5f * ((i == j ? 1.f : 0.f) - *g) : 0.f);
+  }
+  __syncthreads();
+  // V is read as a whole before it is replaced: the product goes to the W area
+  cta_gemm<float>(r, n, r, G, vs ? ldg : r, V, ldv, W, n, false);
+  for (int idx = threadIdx.x; idx < r * n; idx += blockDim.x) {
+    const float v = W[idx];
+    out[idx] = v;
+    if (vs) V[(size_t)(idx / n) * ldv + idx % n] = v;
+  }
+  __syncthreads();
+  cta_gemm_nt<float>(m, r, n, C, n, V, ldv, US, r);
+  for (int idx = threadIdx.x; idx < m * r; idx += blockDim.x)
+    if (sh.sig[sh.perm[idx % r]] * scl <= 1e-12) US[idx] = 0.f;
+  if (threadIdx.x == 0) J.dst.ranks[k] = r;
+  __syncthreads();
+  return r;
+}
+
 // The rounding job as run by the leader CTA of its cluster (the whole job
 // when the cluster has one CTA).
 template <typename T>
@@ -1225,7 +1388,7 @@ __device__ void round_job_body(const RoundJob& J, int L_arg, int n_bits_arg, con
     T* US = scr + J.lay.us_off;
     int r = 0;
     bool done = false;             // randomized truncation accepted
-    bool full64 = false;           // full SVD taken in FP64 (svd64_site)
+    bool full64 = false;           // full SVD taken by svd64_site or svd32_site
     // ---- randomized truncation at a target rank, certified (learned-rank path)
     int tgt = 0;
     if (J.rsvd_mode && lc != nullptr && lc->omega != nullptr) {
@@ -1377,6 +1540,14 @@ __device__ void round_job_body(const RoundJob& J, int L_arg, int n_bits_arg, con
       r = svd64_site<T>(J, L, k, C, m, n, out, US, scr, work, sh, cc, status, lc, pc, delta);
       if (r == 0) return;
       full64 = true;
+    }
+    if constexpr (sizeof(T) == 4) {
+      if (!done && !full64 && svd32_fits(m, n)) {
+        const SiteShared sh{s_red, s_tau, s_sig, s_perm, &s_bad, &s_rank, &s_flops};
+        r = svd32_site(J, L, k, C, m, n, out, US, scr, work, sh, s_wv, blockIdx.x / cc.P, status, lc, pc, delta);
+        if (r == 0) return;
+        full64 = true;
+      }
     }
     if (!done && !full64) {
       if (ncol > MAXK) { if (threadIdx.x == 0) flag(status, ST_CAPACITY); return; }
