@@ -17,6 +17,7 @@
 #include "gemm.cuh"
 #include "tcgemm.cuh"
 #include "linalg.cuh"
+#include "qr_reg.cuh"
 
 namespace tn {
 
@@ -214,8 +215,36 @@ __global__ void env_edges_kernel(const FitJob* __restrict__ jobs, int L) {
   }
 }
 
+static constexpr int FIT_SMEM = 176 * 1024;  // work matrix of the centre shifts and the QR panel
+
+// QR of the m x n matrix that `fill(i, c)` gives, Q (m x kk) and R (kk x n): FP32
+// by the register QR (its panel in shared memory, the matrix beside it where it
+// fits), other shapes and FP64 by the blocked one.  `x`: free scratch of the job
+// (qr_blk_scratch).
+template <typename T, typename F>
+__device__ __forceinline__ void fit_qr(F&& fill, int m, int n, T* Qt, T* Rm, T* qscr, T* x, unsigned char* fsm,
+                                       double* tau, T* wv, double* red) {
+  const bool reg_qr = sizeof(T) == 4 && qr_reg_fits(m, n) && qr_reg_bytes(m) <= (size_t)FIT_SMEM;
+  const size_t wsz = ((size_t)m * (n | 1) * sizeof(T) + 15) & ~(size_t)15;
+  const bool in_smem = wsz + (reg_qr ? qr_reg_bytes(m) : 0) <= (size_t)FIT_SMEM;
+  const int ldw = in_smem ? (n | 1) : n;
+  T* work = in_smem ? (T*)fsm : qscr;
+  for (int idx = threadIdx.x; idx < m * n; idx += blockDim.x) {
+    const int i = idx / n, c = idx % n;
+    work[(size_t)i * ldw + c] = fill(i, c);
+  }
+  __syncthreads();
+  if constexpr (sizeof(T) == 4) {
+    if (reg_qr) {
+      float* V = (float*)(fsm + (in_smem ? wsz : 0));
+      qr_reg(work, m, n, ldw, Qt, imin(m, n), Rm, n, V, V + (size_t)m * 16, x, (float*)tau);
+      return;
+    }
+  }
+  householder_qr_blk<T>(work, m, n, ldw, Qt, imin(m, n), Rm, n, tau, wv, red, x, x + (size_t)m * QB);
+}
+
 // Right-orthogonalise A: LQ at k = L-1..1, A_{k-1} <- A_{k-1} L.
-static constexpr int FIT_SMEM = 96 * 1024;   // work matrix of the centre shifts
 
 template <typename T>
 __global__ void __launch_bounds__(FT) rortho_kernel(const FitJob* __restrict__ jobs, int L,
@@ -232,16 +261,9 @@ __global__ void __launch_bounds__(FT) rortho_kernel(const FitJob* __restrict__ j
     const int a = J.A.ranks[k], a1 = J.A.ranks[k + 1], a0 = J.A.ranks[k - 1];
     const int m = 2 * a1, n = a, kk = imin(m, n);
     if (kk > 1024 || n > 1024) { if (threadIdx.x == 0) atomicOr(status, ST_CAPACITY); return; }
-    const int ldw = ((size_t)m * (n | 1) * sizeof(T) <= (size_t)FIT_SMEM) ? (n | 1) : n;
-    T* work = ((size_t)m * ldw * sizeof(T) <= (size_t)FIT_SMEM) ? (T*)fsm : (T*)J.qscr;
     T* Ak = (T*)J.A.base + core_offset(L, J.A.cap, k);
     T* Ap = (T*)J.A.base + core_offset(L, J.A.cap, k - 1);
-    for (int idx = threadIdx.x; idx < m * n; idx += blockDim.x) {
-      const int i = idx / n, c = idx % n;      // work[i][c] = Ak[c][i]
-      work[(size_t)i * ldw + c] = Ak[(size_t)c * m + i];
-    }
-    __syncthreads();
-    householder_qr_blk<T>(work, m, n, ldw, Qt, kk, Rm, n, tau, wv, red, (T*)J.x, (T*)J.x + (size_t)m * QB);
+    fit_qr<T>([&](int i, int c) { return Ak[(size_t)c * m + i]; }, m, n, Qt, Rm, (T*)J.qscr, (T*)J.x, fsm, tau, wv, red);
     if (ctr && threadIdx.x == 0) atomicAdd(&ctr[C_FIT_QR], qr_flops(m, n) + 2.0 * 2 * a0 * a * kk);
     // A_k <- Qt^T (kk x m) ; A_{k-1} <- A_{k-1} (2a0 x a) * Rm^T (a x kk)
     for (int idx = threadIdx.x; idx < kk * m; idx += blockDim.x) {
@@ -286,16 +308,10 @@ __global__ void __launch_bounds__(FT) shift_centre_kernel(const FitJob* __restri
   const int n = mode == 0 ? a1 : a;
   const int kk = imin(m, n);
   if (kk > 1024 || n > 1024) { if (threadIdx.x == 0) atomicOr(status, ST_CAPACITY); return; }
-  const int ldw = ((size_t)m * (n | 1) * sizeof(T) <= (size_t)FIT_SMEM) ? (n | 1) : n;
-  T* work = ((size_t)m * ldw * sizeof(T) <= (size_t)FIT_SMEM) ? (T*)fsm : (T*)J.qscr;
-  for (int idx = threadIdx.x; idx < m * n; idx += blockDim.x) {
-    const int i = idx / n, col = idx % n;
-    work[(size_t)i * ldw + col] = mode == 0 ? Ab[idx] : Ab[(size_t)col * m + i];
-  }
-  __syncthreads();
-  // blocked QR; its panel scratch is the X buffer (free between the local update and
-  // the environment update)
-  householder_qr_blk<T>(work, m, n, ldw, Qt, kk, Rm, n, tau, wv, red, (T*)J.x, (T*)J.x + (size_t)m * QB);
+  // its scratch is the X buffer (free between the local update and the environment
+  // update)
+  fit_qr<T>([&](int i, int col) { return mode == 0 ? Ab[(size_t)i * n + col] : Ab[(size_t)col * m + i]; }, m, n, Qt, Rm,
+            (T*)J.qscr, (T*)J.x, fsm, tau, wv, red);
   if (ctr && threadIdx.x == 0) atomicAdd(&ctr[C_FIT_QR], qr_flops(m, n));
   if (mode == 0) {
     for (int idx = threadIdx.x; idx < m * kk; idx += blockDim.x) Ac[idx] = Qt[idx];

@@ -653,10 +653,11 @@ namespace tn {
 static constexpr int QB = 16;            // panel width
 static constexpr int QNG = 4;            // row groups of the V^T X products
 
-// Scratch (global or shared): vb >= m * QB, wb >= (QNG + 1) * QB * n elements.
+// Scratch (global or shared): vb >= m * QB, wb >= (QNG + 1) * QB * n elements; or
+// the T factors of qr_reg (QB n + QB^2).
 template <typename T>
 __host__ __device__ inline size_t qr_blk_scratch(int m, int n) {
-  return (size_t)m * QB + (size_t)(QNG + 1) * QB * n;
+  return (size_t)m * QB + (size_t)(QNG + 1) * QB * n + QB * QB;
 }
 
 // V (mr x QB, ld QB) of the panel [p0, pe): unit diagonal, zeros above it,

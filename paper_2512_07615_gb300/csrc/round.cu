@@ -13,6 +13,7 @@
 #include "cluster.cuh"
 #include "jacobi_reg.cuh"
 #include "linalg.cuh"
+#include "qr_reg.cuh"
 
 namespace tn {
 
@@ -1050,12 +1051,17 @@ __host__ __device__ inline size_t svd32_vbytes(int r, int n) {
   return ((size_t)r * (n | 1) + (size_t)r * (r | 1)) * sizeof(float);
 }
 
+// Bytes of the copy of C that svd32_site's QR works on, its panel after it.
+__host__ __device__ inline size_t svd32_qr_off(int m, int n) {
+  return ((size_t)m * (n | 1) * sizeof(float) + 15) & ~(size_t)15;
+}
+
 // Whether svd32_site takes an m x n centre matrix: its vectors fit the register
 // Jacobi, and W with the QR panel (m > n) fits the work area.
 __host__ __device__ inline bool svd32_fits(int m, int n) {
   const int k = m < n ? m : n;
   if (!jacobi_reg_fits(k, n)) return false;
-  if (m > n && (size_t)m * (n | 1) * sizeof(float) > (size_t)SM_WORK) return false;
+  if (m > n && (!qr_reg_fits(m, n) || svd32_qr_off(m, n) + qr_reg_bytes(m) > (size_t)SM_WORK)) return false;
   return (size_t)jacobi_reg_cols(k) * jacobi_reg_ld(n) * sizeof(float) <= (size_t)SM_WORK;
 }
 
@@ -1071,8 +1077,8 @@ __host__ __device__ inline bool svd32_fits(int m, int n) {
 // Leaves singular values and order in sh.sig / sh.perm; returns the kept rank,
 // or 0 after flagging an error.
 __device__ __noinline__ int svd32_site(const RoundJob& J, int L, int k, const float* C, int m, int n, float* out,
-                                       float* US, float* scr, float* work, const SiteShared& sh, float* wv,
-                                       int job, int* status, const LearnCtx* lc, PhaseClock& pc,
+                                       float* US, float* scr, float* work, const SiteShared& sh, int job,
+                                       int* status, const LearnCtx* lc, PhaseClock& pc,
                                        double delta) {
   const int ncol = imin(m, n), ld = jacobi_reg_ld(n), ncp = jacobi_reg_cols(ncol);
   float* W = work;
@@ -1098,10 +1104,8 @@ __device__ __noinline__ int svd32_site(const RoundJob& J, int L, int k, const fl
     for (int idx = threadIdx.x; idx < m * n; idx += blockDim.x) work[(size_t)(idx / n) * lda + idx % n] = C[idx];
     __syncthreads();
     float* R = scr + J.lay.jv_off;
-    float* vb = scr + J.lay.qw_off;
-    householder_qr_blk<float>(work, m, n, lda, nullptr, 0, R, n, sh.tau, wv, sh.red, vb, vb + (size_t)m * QB);
-    if (threadIdx.x == 0) sh.tau[1] = scl;
-    __syncthreads();
+    float* V = (float*)((unsigned char*)work + svd32_qr_off(m, n));
+    qr_reg(work, m, n, lda, nullptr, 0, R, n, V, V + (size_t)m * 16, scr + J.lay.qw_off, (float*)sh.sig);
     X = R;
   }
   for (int idx = threadIdx.x; idx < ncp * ld; idx += blockDim.x) {
@@ -1323,7 +1327,10 @@ __device__ void round_job_body(const RoundJob& J, int L_arg, int n_bits_arg, con
     // (b) M = Rc * blockdiag(W): rows (r, s), row length Rk1, leading dim ld
     const int mrows = 2 * rc;
     int ld = Rk1 | 1;
-    bool in_smem = (size_t)mrows * ld * sizeof(T) <= (size_t)SM_WORK;
+    // FP32: the register QR, with its panel beside M in the work area
+    const bool reg_qr = sizeof(T) == 4 && qr_reg_fits(mrows, Rk1) && qr_reg_bytes(mrows) <= (size_t)SM_WORK;
+    const size_t msz = ((size_t)mrows * ld * sizeof(T) + 15) & ~(size_t)15;
+    bool in_smem = msz + (reg_qr ? qr_reg_bytes(mrows) : 0) <= (size_t)SM_WORK;
     if (!in_smem) ld = Rk1;
     T* M = in_smem ? work : scr + J.lay.m_off;
     const bool last = (k == L - 1);
@@ -1348,11 +1355,17 @@ __device__ void round_job_body(const RoundJob& J, int L_arg, int n_bits_arg, con
     // (c) QR of M (mrows x Rk1) -> Q_k (ld rq), new carried R (rq x Rk1, ld Rk1)
     const int rq = imin(mrows, Rk1);
     if (rq > MAXK || Rk1 > MAXK) { if (threadIdx.x == 0) flag(status, ST_CAPACITY); return; }
-    {
-      T* vb = scr + J.lay.qw_off;
-      householder_qr_blk<T>(M, mrows, Rk1, ld, Qk, rq, Rc, Rk1, s_tau, s_wv, s_red, vb,
-                            vb + (size_t)mrows * QB);
+    T* vb = scr + J.lay.qw_off;
+    bool qr_done = false;
+    if constexpr (sizeof(T) == 4) {
+      if (reg_qr) {
+        float* V = (float*)((unsigned char*)work + (in_smem ? msz : 0));
+        qr_reg(M, mrows, Rk1, ld, Qk, rq, Rc, Rk1, V, V + (size_t)mrows * 16, vb, (float*)s_sig);
+        qr_done = true;
+      }
     }
+    if (!qr_done)
+      householder_qr_blk<T>(M, mrows, Rk1, ld, Qk, rq, Rc, Rk1, s_tau, s_wv, s_red, vb, vb + (size_t)mrows * QB);
     if (threadIdx.x == 0) flops += qr_flops(mrows, Rk1);
     pc.lap(PH_QR);
     rc = rq;
@@ -1544,7 +1557,7 @@ __device__ void round_job_body(const RoundJob& J, int L_arg, int n_bits_arg, con
     if constexpr (sizeof(T) == 4) {
       if (!done && !full64 && svd32_fits(m, n)) {
         const SiteShared sh{s_red, s_tau, s_sig, s_perm, &s_bad, &s_rank, &s_flops};
-        r = svd32_site(J, L, k, C, m, n, out, US, scr, work, sh, s_wv, blockIdx.x / cc.P, status, lc, pc, delta);
+        r = svd32_site(J, L, k, C, m, n, out, US, scr, work, sh, blockIdx.x / cc.P, status, lc, pc, delta);
         if (r == 0) return;
         full64 = true;
       }
