@@ -32,7 +32,8 @@ struct ClusterCmd {
   int op;                 // 0 = exit, 1 = FP64 Jacobi on the job's W64 / V64 (columns in
                           // global memory), 2 = row-partitioned FP64 SVD of site k
   int ncol, len, maxsw;
-  int m, n, k, pad;
+  int m, n, k;
+  int sw32;               // logged FP32 sweeps that start the SVD (-1: their V is in scratch)
   double delta, scl;
 };
 
@@ -242,7 +243,7 @@ __device__ inline bool cl_xchg_wait(ClusterCtx& c) {
 
 // Leader: write a command into every worker's shared memory, then meet them.
 __device__ inline bool cl_command(ClusterCtx& c, int op, int ncol, int len, int maxsw, int m = 0, int n = 0,
-                                  int k = 0, double delta = 0.0, double scl = 0.0) {
+                                  int k = 0, double delta = 0.0, double scl = 0.0, int sw32 = -1) {
   if (c.P == 1) return true;
   if (cl_alive(c) && threadIdx.x >= 1 && threadIdx.x < (unsigned)c.P) {
     const unsigned r = threadIdx.x;
@@ -253,6 +254,7 @@ __device__ inline bool cl_command(ClusterCtx& c, int op, int ncol, int len, int 
     cl_store_remote(&c.sh->cmd.m, r, m);
     cl_store_remote(&c.sh->cmd.n, r, n);
     cl_store_remote(&c.sh->cmd.k, r, k);
+    cl_store_remote(&c.sh->cmd.sw32, r, sw32);
     cl_store_remote(&c.sh->cmd.delta, r, delta);
     cl_store_remote(&c.sh->cmd.scl, r, scl);
   }

@@ -105,6 +105,7 @@ struct RoundLayout {
   size_t q_off[TN_MAXL + 1];  // left-orthogonal cores of the QR sweep
   size_t w_off, m_off, r_off, c_off, jw_off, jv_off, us_off, rz_off, qw_off, total;
   size_t jw64_off, jv64_off;  // FP64 Jacobi matrices (in elements of T; = jw/jv for T = double)
+  size_t log_off;             // rotations of the FP32 sweeps that start an FP64 SVD
 };
 
 // Learned-rank rounding state shared by all jobs of a launch (nullable parts).

@@ -74,9 +74,10 @@ __device__ __forceinline__ bool jr_angle(float& al, float& be, float ga, float t
 
 // One step: the pairs (X[i], Y[(i + S) % B]) of two blocks, their squared norms
 // na (of X[q]) and nb (of Y[q]) kept by lane group q.
-template <int B, int EPL, int S>
+// LOG: lane group q puts the pair's (c, s) at its log.
+template <int B, int EPL, int S, bool LOG>
 __device__ __forceinline__ bool jr_cross(float (&X)[B][EPL], float (&Y)[B][EPL], float& na, float& nb, float tol,
-                                         int lane) {
+                                         int lane, float2* log) {
   constexpr unsigned F = 0xffffffffu;
   constexpr int G = 32 / B;
   float d[B];
@@ -91,6 +92,7 @@ __device__ __forceinline__ bool jr_cross(float (&X)[B][EPL], float (&Y)[B][EPL],
   float be = S == 0 ? nb : __shfl_sync(F, nb, (lane + S * G) & 31);
   float c, s;
   const bool go = jr_angle(na, be, ga, tol, c, s);
+  if (LOG && lane % G == 0) *log = make_float2(c, s);
   if (!__any_sync(F, go)) return false;
   nb = S == 0 ? be : __shfl_sync(F, be, (lane + 32 - S * G) & 31);
 #pragma unroll
@@ -108,8 +110,8 @@ __device__ __forceinline__ bool jr_cross(float (&X)[B][EPL], float (&Y)[B][EPL],
 
 // The pairs inside the two blocks, (X[i0], X[i1]), (X[i2], X[i3]) and the same of
 // Y (B = 4), or (X[0], X[1]) and (Y[0], Y[1]) (B = 2).
-template <int B, int EPL, int I0, int I1, int I2, int I3>
-__device__ __forceinline__ bool jr_inner(float (&X)[B][EPL], float (&Y)[B][EPL], float tol, int lane) {
+template <int B, int EPL, int I0, int I1, int I2, int I3, bool LOG>
+__device__ __forceinline__ bool jr_inner(float (&X)[B][EPL], float (&Y)[B][EPL], float tol, int lane, float2* log) {
   constexpr unsigned F = 0xffffffffu;
   constexpr int G = 32 / B, H = B / 2;
   float d[B], na[B], nb[B];
@@ -131,6 +133,7 @@ __device__ __forceinline__ bool jr_inner(float (&X)[B][EPL], float (&Y)[B][EPL],
   const float ga = jr_reduce<B>(d, lane);
   float al = jr_reduce<B>(na, lane), be = jr_reduce<B>(nb, lane), c, s;
   const bool go = jr_angle(al, be, ga, tol, c, s);
+  if (LOG && lane % G == 0) *log = make_float2(c, s);
   if (!__any_sync(F, go)) return false;
 #pragma unroll
   for (int q = 0; q < B; ++q) {
@@ -184,9 +187,16 @@ __device__ __forceinline__ void jr_load(const float* p, float (&X)[B][EPL], int 
 // count and length, columns padded to a multiple of 2 B), at most maxsw.  Returns
 // the sweeps that rotated anything (maxsw if the last one still did).  W is the
 // exchange buffer meanwhile: 2 W blocks are one block out and one block in per
-// warp, so a sending phase alternates between its halves.
-template <int B, int EPL>
-__device__ __noinline__ int jacobi_reg_run(float* W, int ncol, int len, int maxsw) {
+// warp, so a sending phase alternates between its halves.  A sweep reverses the
+// blocks; they are stored back in their first order.
+// log (LOG) receives the (c, s) of every pair of every sweep,
+// log[((sweep * jr_steps + step) * B + q) * nw + w] for pair q of warp w, which
+// jacobi_reg_apply reads.
+template <int B>
+__host__ __device__ constexpr int jr_steps(int nw) { return B - 1 + 2 * nw * B; }
+
+template <int B, int EPL, bool LOG>
+__device__ __noinline__ int jacobi_reg_run(float* W, int ncol, int len, int maxsw, float2* log) {
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   const int nw = (ncol + 2 * B - 1) / (2 * B);              // warps that hold columns
   constexpr int BS = B * 32 * EPL;                          // floats of a block
@@ -201,6 +211,9 @@ __device__ __noinline__ int jacobi_reg_run(float* W, int ncol, int len, int maxs
     jr_load<B, EPL>(W + (size_t)(2 * wid + 1) * BS, Y, lane);
     float* buf[2] = {W, W + (size_t)nw * BS};
     auto meet = [&]() { asm volatile("bar.sync 1, %0;" ::"r"(nw * 32) : "memory"); };
+    const int lstep = B * nw;
+    float2* lg = log + (LOG ? (size_t)(lane / (32 / B)) * nw + wid : 0);
+    auto next = [&]() { if (LOG) lg += lstep; };
     // all cross pairs of the two blocks, with norms taken afresh
     auto cross = [&]() -> bool {
       float na[B], nb[B];
@@ -216,11 +229,17 @@ __device__ __noinline__ int jacobi_reg_run(float* W, int ncol, int len, int maxs
         nb[i] = b;
       }
       float al = jr_reduce<B>(na, lane), be = jr_reduce<B>(nb, lane);
-      bool r = jr_cross<B, EPL, 0>(X, Y, al, be, tol, lane);
-      if constexpr (B >= 2) r |= jr_cross<B, EPL, 1>(X, Y, al, be, tol, lane);
+      bool r = jr_cross<B, EPL, 0, LOG>(X, Y, al, be, tol, lane, lg);
+      next();
+      if constexpr (B >= 2) {
+        r |= jr_cross<B, EPL, 1, LOG>(X, Y, al, be, tol, lane, lg);
+        next();
+      }
       if constexpr (B == 4) {
-        r |= jr_cross<B, EPL, 2>(X, Y, al, be, tol, lane);
-        r |= jr_cross<B, EPL, 3>(X, Y, al, be, tol, lane);
+        r |= jr_cross<B, EPL, 2, LOG>(X, Y, al, be, tol, lane, lg);
+        next();
+        r |= jr_cross<B, EPL, 3, LOG>(X, Y, al, be, tol, lane, lg);
+        next();
       }
       return r;
     };
@@ -228,11 +247,15 @@ __device__ __noinline__ int jacobi_reg_run(float* W, int ncol, int len, int maxs
     for (; sweep < maxsw; ++sweep) {
       bool rot = false;
       if constexpr (B == 4) {
-        rot |= jr_inner<B, EPL, 0, 1, 2, 3>(X, Y, tol, lane);
-        rot |= jr_inner<B, EPL, 0, 2, 1, 3>(X, Y, tol, lane);
-        rot |= jr_inner<B, EPL, 0, 3, 1, 2>(X, Y, tol, lane);
+        rot |= jr_inner<B, EPL, 0, 1, 2, 3, LOG>(X, Y, tol, lane, lg);
+        next();
+        rot |= jr_inner<B, EPL, 0, 2, 1, 3, LOG>(X, Y, tol, lane, lg);
+        next();
+        rot |= jr_inner<B, EPL, 0, 3, 1, 2, LOG>(X, Y, tol, lane, lg);
+        next();
       } else if constexpr (B == 2) {
-        rot |= jr_inner<B, EPL, 0, 1, 0, 1>(X, Y, tol, lane);
+        rot |= jr_inner<B, EPL, 0, 1, 0, 1, LOG>(X, Y, tol, lane, lg);
+        next();
       }
       for (int ph = 0; ph < nw; ++ph) {
         // even phase; the blocks trade places: Y (now first) goes to the left
@@ -247,6 +270,7 @@ __device__ __noinline__ int jacobi_reg_run(float* W, int ncol, int len, int maxs
           rot |= cross();
           jr_store<B, EPL>(buf[1] + (size_t)(wid + 1) * BS, X, lane);
         } else {
+          if (LOG) lg += B * lstep;                          // no pairs here: the log has a gap
           jr_store<B, EPL>(buf[1], Y, lane);
 #pragma unroll
           for (int i = 0; i < B; ++i)
@@ -263,8 +287,10 @@ __device__ __noinline__ int jacobi_reg_run(float* W, int ncol, int len, int maxs
       meet();
       if (!any) break;
     }
-    jr_store<B, EPL>(W + (size_t)(2 * wid) * BS, X, lane);
-    jr_store<B, EPL>(W + (size_t)(2 * wid + 1) * BS, Y, lane);
+    const int done = sweep < maxsw ? sweep + 1 : sweep;     // the last one rotated nothing
+    const int px = done & 1 ? 2 * nw - 1 - 2 * wid : 2 * wid, py = done & 1 ? px - 1 : px + 1;
+    jr_store<B, EPL>(W + (size_t)px * BS, X, lane);
+    jr_store<B, EPL>(W + (size_t)py * BS, Y, lane);
   }
   __shared__ int s_sweeps;
   if (threadIdx.x == 0) s_sweeps = sweep;
@@ -288,15 +314,142 @@ __host__ __device__ inline int jacobi_reg_cols(int ncol) {
 // One-sided FP32 Jacobi of the padded columns in W (see jacobi_reg_run).  Blocks
 // of 4 columns when more than 64 are there, of 2 or 1 below so that all 16 warps
 // have columns.
-__device__ __forceinline__ int jacobi_reg(float* W, int ncol, int len, int maxsw) {
+template <bool LOG>
+__device__ __forceinline__ int jacobi_reg(float* W, int ncol, int len, int maxsw, float2* log) {
   const int b = jacobi_reg_block(ncol);
-#define JR(B)                                                                   \
-  (len <= 32    ? jacobi_reg_run<B, 1>(W, ncol, len, maxsw)                     \
-   : len <= 64  ? jacobi_reg_run<B, 2>(W, ncol, len, maxsw)                     \
-   : len <= 128 ? jacobi_reg_run<B, 4>(W, ncol, len, maxsw)                     \
-                : jacobi_reg_run<B, 8>(W, ncol, len, maxsw))
-  return b == 1 ? JR(1) : b == 2 ? JR(2) : JR(4);
+#define JR(B, LOG)                                                              \
+  (len <= 32    ? jacobi_reg_run<B, 1, LOG>(W, ncol, len, maxsw, log)           \
+   : len <= 64  ? jacobi_reg_run<B, 2, LOG>(W, ncol, len, maxsw, log)           \
+   : len <= 128 ? jacobi_reg_run<B, 4, LOG>(W, ncol, len, maxsw, log)           \
+                : jacobi_reg_run<B, 8, LOG>(W, ncol, len, maxsw, log))
+  return b == 1 ? JR(1, LOG) : b == 2 ? JR(2, LOG) : JR(4, LOG);
 #undef JR
+}
+
+// Pairs of a sweep's log, and the sweeps that are logged at most (the ones that
+// an FP32 Jacobi needs are about ten; what is left at the limit is the FP64
+// sweeps' work).
+static constexpr int JR_LOG_SWEEPS = 16;
+__host__ __device__ inline size_t jacobi_reg_log_sweep(int ncol) {
+  const int b = jacobi_reg_block(ncol), nw = (ncol + 2 * b - 1) / (2 * b);
+  return (size_t)(b - 1 + 2 * nw * b) * b * nw;
+}
+
+// Rows [r0, r0 + nr) of the product J of the logged rotations (J = I before), as
+// entries of its columns: out[c * ld + r] for c, r < ncol.  Rows of J are
+// independent, so the CTAs of a cluster share them.  A half-warp holds a row: its
+// lane w the columns that warp w of jacobi_reg_run held, and passes them on to its
+// neighbours as that warp did.  A sweep of the log is staged in shared memory (st,
+// two sweeps long) while the one before is applied.  ~40 cycles a step, the latency
+// of its dependent rotations.
+template <int B>
+__device__ __noinline__ void jacobi_reg_apply_run(const float2* log, int sweeps, int ncol, int r0, int nr, float* out,
+                                                  int ld, float2* st) {
+  constexpr unsigned F = 0xffffffffu;
+  const int nw = (ncol + 2 * B - 1) / (2 * B), per = B * nw, size = jr_steps<B>(nw) * per;
+  const int w = threadIdx.x & 15, hw = threadIdx.x >> 4, nhw = blockDim.x >> 4;
+  const int lane = threadIdx.x & 31, half = lane & 16;
+  const int wl = imin(w, nw - 1);
+  const int left = half | (w == 0 ? nw - 1 : w - 1), right = half | (w == nw - 1 ? 0 : imin(w + 1, 15));
+  const bool last = w + 1 >= nw;
+  auto stage = [&](int sw) {
+    const float2* lg = log + (size_t)sw * size;
+    float2* d = st + (size_t)(sw & 1) * size;
+    // 16 bytes (`size` is even) past L1, which may hold an earlier site's log
+    for (int i = 2 * threadIdx.x; i < size; i += 2 * blockDim.x)
+      asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((unsigned)__cvta_generic_to_shared(d + i)), "l"(lg + i)
+                   : "memory");
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  };
+  auto rot = [](float& x, float& y, float2 g) {
+    const float u = g.x * x - g.y * y, v = g.y * x + g.x * y;
+    x = u;
+    y = v;
+  };
+  for (int base = r0; base < r0 + nr; base += nhw) {
+    const int row = base + hw;
+    float X[B], Y[B];
+#pragma unroll
+    for (int i = 0; i < B; ++i) {
+      X[i] = (2 * w) * B + i == row ? 1.f : 0.f;
+      Y[i] = (2 * w + 1) * B + i == row ? 1.f : 0.f;
+    }
+    if (sweeps > 0) stage(0);
+    for (int sw = 0; sw < sweeps; ++sw) {
+      if (sw + 1 < sweeps) {
+        stage(sw + 1);
+        asm volatile("cp.async.wait_group 1;" ::: "memory");
+      } else {
+        asm volatile("cp.async.wait_group 0;" ::: "memory");
+      }
+      __syncthreads();
+      if ((hw & ~1) + base < r0 + nr) {                      // the warp holds a row
+        const float2* p = st + (size_t)(sw & 1) * size + wl;
+        float2 g[B];
+        auto get = [&]() {
+#pragma unroll
+          for (int q = 0; q < B; ++q) g[q] = p[q * nw];
+          p += per;
+        };
+        if constexpr (B == 4) {
+          get(); rot(X[0], X[1], g[0]); rot(X[2], X[3], g[1]); rot(Y[0], Y[1], g[2]); rot(Y[2], Y[3], g[3]);
+          get(); rot(X[0], X[2], g[0]); rot(X[1], X[3], g[1]); rot(Y[0], Y[2], g[2]); rot(Y[1], Y[3], g[3]);
+          get(); rot(X[0], X[3], g[0]); rot(X[1], X[2], g[1]); rot(Y[0], Y[3], g[2]); rot(Y[1], Y[2], g[3]);
+        } else if constexpr (B == 2) {
+          get(); rot(X[0], X[1], g[0]); rot(Y[0], Y[1], g[1]);
+        }
+        float2 e[B][B], o[B][B];                             // the phase's pairs, loaded ahead
+        auto fetch = [&](float2 (&f)[B][B]) {
+#pragma unroll
+          for (int S = 0; S < B; ++S)
+#pragma unroll
+            for (int q = 0; q < B; ++q) f[S][q] = p[(S * B + q) * nw];
+          p += B * per;
+        };
+        fetch(e);
+        for (int ph = 0; ph < nw; ++ph) {
+          fetch(o);
+#pragma unroll
+          for (int S = 0; S < B; ++S)
+#pragma unroll
+            for (int i = 0; i < B; ++i) rot(X[i], Y[(i + S) % B], e[S][i]);
+#pragma unroll
+          for (int i = 0; i < B; ++i) Y[i] = __shfl_sync(F, Y[i], right);
+          if (ph + 1 < nw) fetch(e);
+#pragma unroll
+          for (int S = 0; S < B; ++S)
+#pragma unroll
+            for (int i = 0; i < B; ++i) rot(X[i], Y[(i + S) % B], last ? make_float2(1.f, 0.f) : o[S][i]);
+#pragma unroll
+          for (int i = 0; i < B; ++i) {
+            // the last lane's X is the last position and stays as Y; its Y is the first
+            const float give = last ? Y[i] : X[i], stay = last ? X[i] : Y[i];
+            X[i] = __shfl_sync(F, give, left);
+            Y[i] = stay;
+          }
+        }
+      }
+      __syncthreads();                                       // st is refilled two sweeps on
+    }
+    if (row < r0 + nr && w < nw) {
+      const int px = sweeps & 1 ? 2 * nw - 1 - 2 * w : 2 * w, py = sweeps & 1 ? px - 1 : px + 1;
+#pragma unroll
+      for (int i = 0; i < B; ++i) {
+        if (px * B + i < ncol) __stcg(out + (size_t)(px * B + i) * ld + row, X[i]);
+        if (py * B + i < ncol) __stcg(out + (size_t)(py * B + i) * ld + row, Y[i]);
+      }
+    }
+  }
+  __syncthreads();
+}
+
+// st: shared memory of 2 jacobi_reg_log_sweep(ncol) pairs.
+__device__ __forceinline__ void jacobi_reg_apply(const float2* log, int sweeps, int ncol, int r0, int nr, float* out,
+                                                 int ld, float2* st) {
+  const int b = jacobi_reg_block(ncol);
+  if (b == 1) jacobi_reg_apply_run<1>(log, sweeps, ncol, r0, nr, out, ld, st);
+  else if (b == 2) jacobi_reg_apply_run<2>(log, sweeps, ncol, r0, nr, out, ld, st);
+  else jacobi_reg_apply_run<4>(log, sweeps, ncol, r0, nr, out, ld, st);
 }
 
 }  // namespace tn

@@ -657,7 +657,8 @@ static constexpr int QNG = 4;            // row groups of the V^T X products
 // the T factors of qr_reg (QB n + QB^2).
 template <typename T>
 __host__ __device__ inline size_t qr_blk_scratch(int m, int n) {
-  return (size_t)m * QB + (size_t)(QNG + 1) * QB * n + QB * QB;
+  const size_t panels = (size_t)m * QB + (size_t)(QNG + 1) * QB * n, tf = (size_t)QB * n + QB * QB;
+  return panels > tf ? panels : tf;
 }
 
 // V (mr x QB, ld QB) of the panel [p0, pe): unit diagonal, zeros above it,

@@ -91,6 +91,10 @@ void plan_round_job(RoundJob& j, int L, int n_bits, size_t eb) {
     }
     j.lay.jw64_off = al(2 * w64);
     j.lay.jv64_off = al(2 * v64);
+    size_t lg = 0;                                 // float pairs
+    for (int k = 0; k < L; ++k)
+      lg = std::max(lg, jacobi_reg_log_sweep(imin(imin(j.qb[k], 2 * imin(j.chi, j.qb[k + 1])), 128)));
+    j.lay.log_off = al(2 * lg * JR_LOG_SWEEPS);
   } else {
     j.lay.jw64_off = j.lay.jv64_off = 0;
   }
@@ -696,8 +700,10 @@ __device__ inline void rows_xv(const RowsLayout& R, unsigned char* wa, const T* 
 // [c len / P, (c+1) len / P) of every column of W and [c ncol / P,
 // (c+1) ncol / P) of every column of V.  Every CTA sums the exchanged parts
 // in the same order, so every CTA takes the same rotations.
-// FP32 data (T = float): the leader has already run FP32 sweeps on X alone
-// and left their V0 (FP32, ncol x ncol) in the job's scratch; one FP64
+// FP32 data (T = float): the leader has already run FP32 sweeps on X alone and
+// logged their rotations (sw32 sweeps; every CTA forms its rows of their product
+// V0 from the log), or, with sw32 < 0, left V0 (FP32, ncol x ncol) in the job's
+// scratch; one FP64
 // Newton-Schulz step, spread over the CTAs by blocks of columns, makes it
 // orthogonal to FP64 working accuracy (V0^T V0 - I ~ 1e-6 becomes ~1e-12),
 // W = X V is formed in FP64 and the FP64 sweeps start from there -- the
@@ -711,7 +717,7 @@ __device__ inline void rows_xv(const RowsLayout& R, unsigned char* wa, const T* 
 // sweeps, whether their limit was reached, and the FP64 FLOPs executed.
 template <typename T>
 __device__ int svd64_rows(ClusterCtx& cc, const RoundJob& J, int L, int k, int m, int n, double scl, double delta,
-                          int maxsw, int* sweeps_out, bool* noconv, double* exec_flops = nullptr,
+                          int maxsw, int sw32, int* sweeps_out, bool* noconv, double* exec_flops = nullptr,
                           double* phase_acc = nullptr) {
   constexpr bool two_phase = sizeof(T) == 4;
   extern __shared__ __align__(16) unsigned char smem[];
@@ -736,8 +742,13 @@ __device__ int svd64_rows(ClusterCtx& cc, const RoundJob& J, int L, int k, int m
   double* W = Wl;
   if constexpr (two_phase) {
     const long long t0 = clock64();
-    const float* V0 = (const float*)(scr + J.lay.jv_off);
+    float* V0 = (float*)(scr + J.lay.jv_off);
     const int ld0 = jacobi_ld<float>(ncol), ld1 = jacobi_ld<double>(ncol);
+    if (sw32 >= 0) {
+      // this CTA's rows of V0 from the leader's log
+      jacobi_reg_apply((const float2*)(scr + J.lay.log_off), sw32, ncol, v0, vi, V0, ld0, (float2*)wa);
+      cl_sync(cc);
+    }
     double* V1 = (double*)(scr + J.lay.jv64_off);
     rows_ns_step<float>(R, wa, V0, ld0, V1, ld1, ncol, v0, vi);
     cl_sync(cc);                                  // every block of V1 written (cluster-scope fence)
@@ -893,35 +904,55 @@ __device__ __noinline__ int svd64_site(const RoundJob& J, int L, int k, const T*
   if (!in_smem && cc.P > 1 && rows_layout(ncol, len, cc.P, sizeof(T) == 4).total <= (size_t)SM_WORK) {
     // rows of the Jacobi matrices spread over the cluster, in shared memory
     pc.lap(PH_SVD_OUT);
+    int sw32 = 0;
+    bool logged = false;
     if constexpr (sizeof(T) == 4) {
-      // FP32 data: FP32 sweeps on X by this CTA alone (the in-CTA Jacobi of the
-      // FP32 path; its own stopping rule, at most 30 sweeps, convergence not
-      // required), V0 left in the job's scratch for the cluster
-      const int ldw32 = jacobi_ld<float>(len), ldv32 = jacobi_ld<float>(ncol);
-      const size_t need32 = ((size_t)ncol * ldw32 + (size_t)ncol * ldv32) * sizeof(float);
-      float* Vg = (float*)(scr + J.lay.jv_off);
-      // W (the hot operand: len entries per rotated column) in shared memory
-      // whenever it fits there alone; V with it if both fit, else in scratch
-      const bool w_smem = (size_t)ncol * ldw32 * sizeof(float) <= (size_t)SM_WORK;
-      float* Wf = w_smem ? (float*)work : (float*)(scr + J.lay.jw_off);
-      float* Vf = need32 <= (size_t)SM_WORK ? (float*)work + (size_t)ncol * ldw32 : Vg;
-      for (int idx = threadIdx.x; idx < ncol * len; idx += blockDim.x) {
-        const int jj = idx / len, i = idx % len;
-        Wf[(size_t)jj * ldw32 + i] = (float)(scl * (double)(trans ? C[(size_t)i * n + jj] : C[(size_t)jj * n + i]));
+      // FP32 data: FP32 sweeps on X by this CTA alone (its own stopping rule, a
+      // sweep limit, convergence not required).  In registers where X fits: W only,
+      // the rotations logged for the cluster to form V0 (a row of V0 per half-warp,
+      // ~1/16 of the sweeps' time on 16 CTAs, where carrying V along would double
+      // the sweeps' work)
+      if (jacobi_reg_fits(ncol, len)) {
+        float* Wf = (float*)work;
+        const int ldw32 = jacobi_reg_ld(len), ncp = jacobi_reg_cols(ncol);
+        for (int idx = threadIdx.x; idx < ncp * ldw32; idx += blockDim.x) {
+          const int jj = idx / ldw32, i = idx % ldw32;
+          Wf[idx] = jj < ncol && i < len ? (float)(scl * (double)(trans ? C[(size_t)i * n + jj] : C[(size_t)jj * n + i]))
+                                         : 0.f;
+        }
+        __syncthreads();
+        sw32 = jacobi_reg<true>(Wf, ncol, len, imin(maxsw, JR_LOG_SWEEPS), (float2*)(scr + J.lay.log_off));
+        logged = true;
+        __threadfence();                          // the log, before the workers are told of it
+      } else {
+        // larger: the in-CTA Jacobi of the FP32 path, V0 left in the job's scratch
+        const int ldw32 = jacobi_ld<float>(len), ldv32 = jacobi_ld<float>(ncol);
+        const size_t need32 = ((size_t)ncol * ldw32 + (size_t)ncol * ldv32) * sizeof(float);
+        float* Vg = (float*)(scr + J.lay.jv_off);
+        // W (the hot operand: len entries per rotated column) in shared memory
+        // whenever it fits there alone; V with it if both fit, else in scratch
+        const bool w_smem = (size_t)ncol * ldw32 * sizeof(float) <= (size_t)SM_WORK;
+        float* Wf = w_smem ? (float*)work : (float*)(scr + J.lay.jw_off);
+        float* Vf = need32 <= (size_t)SM_WORK ? (float*)work + (size_t)ncol * ldw32 : Vg;
+        for (int idx = threadIdx.x; idx < ncol * len; idx += blockDim.x) {
+          const int jj = idx / len, i = idx % len;
+          Wf[(size_t)jj * ldw32 + i] = (float)(scl * (double)(trans ? C[(size_t)i * n + jj] : C[(size_t)jj * n + i]));
+        }
+        __syncthreads();
+        sw32 = jacobi_cols_fast<float>(Wf, ldw32, Vf, ldv32, ncol, len, imin(maxsw, 30));
+        if (Vf != Vg)
+          for (int idx = threadIdx.x; idx < ncol * ldv32; idx += blockDim.x) __stcg(Vg + idx, Vf[idx]);
+        __syncthreads();
       }
-      __syncthreads();
-      const int sw32 = jacobi_cols_fast<float>(Wf, ldw32, Vf, ldv32, ncol, len, imin(maxsw, 30));
-      if (Vf != Vg)
-        for (int idx = threadIdx.x; idx < ncol * ldv32; idx += blockDim.x) __stcg(Vg + idx, Vf[idx]);
-      __syncthreads();
       if (threadIdx.x == 0) pc.acc[PH_SWEEPS32] += sw32;
       pc.lap(PH_J32);
     }
-    cl_command(cc, 2, ncol, len, maxsw, m, n, k, delta, scl);
+    cl_command(cc, 2, ncol, len, maxsw, m, n, k, delta, scl, logged ? sw32 : -1);
     int sw = 0;
     bool noconv = false;
     double xfl = 0.0;
-    const int r = svd64_rows<T>(cc, J, L, k, m, n, scl, delta, maxsw, &sw, &noconv, &xfl, pc.on ? pc.acc : nullptr);
+    const int r = svd64_rows<T>(cc, J, L, k, m, n, scl, delta, maxsw, logged ? sw32 : -1, &sw, &noconv, &xfl,
+                                pc.on ? pc.acc : nullptr);
     pc.lap(PH_JACOBI);
     if (threadIdx.x == 0) { pc.acc[PH_SVD64_FLOPS] += svd_flops(m, n); pc.acc[PH_SVD64_EXEC] += xfl; }
     const RowsLayout R = rows_layout(ncol, len, cc.P, sizeof(T) == 4);
@@ -1115,7 +1146,7 @@ __device__ __noinline__ int svd32_site(const RoundJob& J, int L, int k, const fl
   __syncthreads();
   const int maxsw = J.max_sweeps > 0 ? J.max_sweeps : 60;
   pc.lap(PH_SVD_OUT);
-  const int sw = jacobi_reg(W, ncol, n, maxsw);
+  const int sw = jacobi_reg<false>(W, ncol, n, maxsw, nullptr);
   pc.lap(PH_JACOBI);
   if (threadIdx.x == 0) {
     pc.acc[6] += sw; pc.acc[7] += 1.0;
@@ -1758,7 +1789,7 @@ __device__ void round_worker(const RoundJob& J, int L_arg, ClusterCtx& cc) {
     if (!cl_sync(cc)) break;
     const volatile ClusterCmd* cmd = (const volatile ClusterCmd*)&cc.sh->cmd;
     const int op = cmd->op, ncol = cmd->ncol, len = cmd->len, maxsw = cmd->maxsw;
-    const int m = cmd->m, n = cmd->n, k = cmd->k;
+    const int m = cmd->m, n = cmd->n, k = cmd->k, sw32 = cmd->sw32;
     const double delta = cmd->delta, scl = cmd->scl;
     __syncthreads();
     if (op == 1) {
@@ -1766,7 +1797,7 @@ __device__ void round_worker(const RoundJob& J, int L_arg, ClusterCtx& cc) {
     } else if (op == 2) {
       int sw = 0;
       bool noconv = false;
-      svd64_rows<T>(cc, J, L, k, m, n, scl, delta, maxsw, &sw, &noconv);
+      svd64_rows<T>(cc, J, L, k, m, n, scl, delta, maxsw, sw32, &sw, &noconv);
     } else {
       break;
     }
