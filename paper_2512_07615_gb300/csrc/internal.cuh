@@ -105,7 +105,9 @@ struct RoundLayout {
   size_t q_off[TN_MAXL + 1];  // left-orthogonal cores of the QR sweep
   size_t w_off, m_off, r_off, c_off, jw_off, jv_off, us_off, rz_off, qw_off, total;
   size_t jw64_off, jv64_off;  // FP64 Jacobi matrices (in elements of T; = jw/jv for T = double)
-  size_t log_off;             // rotations of the FP32 sweeps that start an FP64 SVD
+  // refined FP64 SVDs (RoundJob::refine): rotations of the FP32 sweeps, their
+  // product (floats), a second V with the column norms and the CTAs' maxima
+  size_t log_off, j32_off, vb64_off;
 };
 
 // Learned-rank rounding state shared by all jobs of a launch (nullable parts).
@@ -154,6 +156,7 @@ struct RoundJob {
   int L, n_bits;              // chain length and bits per axis of this job, or 0 = launch's
   double* discard;            // accumulator of squared discarded tails (device), or null
   int svd64;                  // 1: centre SVDs in FP64 on FP32 data (precision TNLBM_MIXED)
+  int refine;                 // 1: scratch for refined FP64 SVDs (launches with clusters)
   int max_sweeps;             // Jacobi sweep limit (0 = 60)
   long long wait_ns;          // limit of every cross-CTA wait in ns (0 = 5 s)
 };
@@ -174,8 +177,9 @@ __host__ __device__ inline int term_bond_bound(const Term& t, int L, int n_bits,
   return 0;
 }
 
-// Fill rw/qb bounds and the scratch layout of a job (host side); j.svd64 must
-// be set before (it adds the FP64 Jacobi matrices for FP32 data).
+// Fill rw/qb bounds and the scratch layout of a job (host side); j.svd64 and
+// j.refine must be set before (they add the FP64 Jacobi matrices for FP32 data,
+// and what the refinement of an FP64 SVD keeps).
 void plan_round_job(RoundJob& j, int L, int n_bits, size_t elem_bytes);
 
 // ------------------------------------------------------------ error helpers

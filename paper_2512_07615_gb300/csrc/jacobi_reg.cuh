@@ -197,10 +197,13 @@ __host__ __device__ constexpr int jr_steps(int nw) { return B - 1 + 2 * nw * B; 
 
 template <int B, int EPL, bool LOG>
 __device__ __noinline__ int jacobi_reg_run(float* W, int ncol, int len, int maxsw, float2* log) {
+  __builtin_assume(__isShared(W));
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   const int nw = (ncol + 2 * B - 1) / (2 * B);              // warps that hold columns
   constexpr int BS = B * 32 * EPL;                          // floats of a block
-  const float tol = 16.f * Eps<float>::v * sqrtf((float)len);
+  // a few ulps above the round-off of a fresh pair; as a start for a refinement
+  // (LOG), which wants small cosines, closer to it
+  const float tol = (LOG ? 4.f : 16.f) * Eps<float>::v * sqrtf((float)len);
   __shared__ int s_rot[2];
   if (threadIdx.x < 2) s_rot[threadIdx.x] = 0;
   __syncthreads();
@@ -342,9 +345,13 @@ __host__ __device__ inline size_t jacobi_reg_log_sweep(int ncol) {
 // neighbours as that warp did.  A sweep of the log is staged in shared memory (st,
 // two sweeps long) while the one before is applied.  ~40 cycles a step, the latency
 // of its dependent rotations.
-template <int B>
-__device__ __noinline__ void jacobi_reg_apply_run(const float2* log, int sweeps, int ncol, int r0, int nr, float* out,
+template <typename O> __device__ __forceinline__ O jr_out(float v) { return (O)v; }
+template <> __device__ __forceinline__ float2 jr_out<float2>(float v) { return make_float2(v, 0.f); }   // v as a pair
+
+template <int B, typename O>
+__device__ __noinline__ void jacobi_reg_apply_run(const float2* log, int sweeps, int ncol, int r0, int nr, O* out,
                                                   int ld, float2* st) {
+  __builtin_assume(__isShared(st));
   constexpr unsigned F = 0xffffffffu;
   const int nw = (ncol + 2 * B - 1) / (2 * B), per = B * nw, size = jr_steps<B>(nw) * per;
   const int w = threadIdx.x & 15, hw = threadIdx.x >> 4, nhw = blockDim.x >> 4;
@@ -435,8 +442,8 @@ __device__ __noinline__ void jacobi_reg_apply_run(const float2* log, int sweeps,
       const int px = sweeps & 1 ? 2 * nw - 1 - 2 * w : 2 * w, py = sweeps & 1 ? px - 1 : px + 1;
 #pragma unroll
       for (int i = 0; i < B; ++i) {
-        if (px * B + i < ncol) __stcg(out + (size_t)(px * B + i) * ld + row, X[i]);
-        if (py * B + i < ncol) __stcg(out + (size_t)(py * B + i) * ld + row, Y[i]);
+        if (px * B + i < ncol) __stcg(out + (size_t)(px * B + i) * ld + row, jr_out<O>(X[i]));
+        if (py * B + i < ncol) __stcg(out + (size_t)(py * B + i) * ld + row, jr_out<O>(Y[i]));
       }
     }
   }
@@ -444,12 +451,13 @@ __device__ __noinline__ void jacobi_reg_apply_run(const float2* log, int sweeps,
 }
 
 // st: shared memory of 2 jacobi_reg_log_sweep(ncol) pairs.
-__device__ __forceinline__ void jacobi_reg_apply(const float2* log, int sweeps, int ncol, int r0, int nr, float* out,
+template <typename O>
+__device__ __forceinline__ void jacobi_reg_apply(const float2* log, int sweeps, int ncol, int r0, int nr, O* out,
                                                  int ld, float2* st) {
   const int b = jacobi_reg_block(ncol);
-  if (b == 1) jacobi_reg_apply_run<1>(log, sweeps, ncol, r0, nr, out, ld, st);
-  else if (b == 2) jacobi_reg_apply_run<2>(log, sweeps, ncol, r0, nr, out, ld, st);
-  else jacobi_reg_apply_run<4>(log, sweeps, ncol, r0, nr, out, ld, st);
+  if (b == 1) jacobi_reg_apply_run<1, O>(log, sweeps, ncol, r0, nr, out, ld, st);
+  else if (b == 2) jacobi_reg_apply_run<2, O>(log, sweeps, ncol, r0, nr, out, ld, st);
+  else jacobi_reg_apply_run<4, O>(log, sweeps, ncol, r0, nr, out, ld, st);
 }
 
 }  // namespace tn

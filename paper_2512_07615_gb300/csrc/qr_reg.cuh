@@ -151,9 +151,13 @@ __host__ __device__ inline bool qr_reg_fits(int m, int n) { return m <= 2 * QRT 
 // V and part: shared memory of qr_reg_vbytes(m) and QR_PART_BYTES; Tg:
 // 16 n + 256 floats (any memory) that keep the T factors for the Q pass; sm: 4 KB
 // of shared memory.  Called by all QRT threads of the block.
-template <int RP>
+template <int RP, bool SH>
 __device__ __noinline__ void qr_reg_run(float* A, int m, int n, int lda, float* Q, int ldq, float* R, int ldr, float* V,
                                         float* part, float* Tg, float* sm) {
+  __builtin_assume(__isShared(V));
+  __builtin_assume(__isShared(part));
+  __builtin_assume(__isShared(sm));
+  if (SH) __builtin_assume(__isShared(A));
   float (*sT)[17] = (float (*)[17])sm;
   float (*s_part)[16][16] = (float (*)[16][16])(sm + 272);
   float (*s_row)[16] = (float (*)[16])(sm + 784);
@@ -314,8 +318,9 @@ __device__ __noinline__ void qr_reg_run(float* A, int m, int n, int lda, float* 
 
 __device__ __forceinline__ void qr_reg(float* A, int m, int n, int lda, float* Q, int ldq, float* R, int ldr, float* V,
                                        float* part, float* Tg, float* sm) {
-  if (m <= QRT) qr_reg_run<1>(A, m, n, lda, Q, ldq, R, ldr, V, part, Tg, sm);
-  else qr_reg_run<2>(A, m, n, lda, Q, ldq, R, ldr, V, part, Tg, sm);
+  if (m <= QRT && __isShared(A)) qr_reg_run<1, true>(A, m, n, lda, Q, ldq, R, ldr, V, part, Tg, sm);
+  else if (m <= QRT) qr_reg_run<1, false>(A, m, n, lda, Q, ldq, R, ldr, V, part, Tg, sm);
+  else qr_reg_run<2, false>(A, m, n, lda, Q, ldq, R, ldr, V, part, Tg, sm);
 }
 
 }  // namespace tn

@@ -9,11 +9,13 @@
 // canonical centre back to site 0 with SVDs (Eq. svd-move) and truncates at the
 // centre to chi / eps.
 #include <algorithm>
+#include <type_traits>
 
 #include "cluster.cuh"
 #include "jacobi_reg.cuh"
 #include "linalg.cuh"
 #include "qr_reg.cuh"
+#include "refine64.cuh"
 
 namespace tn {
 
@@ -91,12 +93,21 @@ void plan_round_job(RoundJob& j, int L, int n_bits, size_t eb) {
     }
     j.lay.jw64_off = al(2 * w64);
     j.lay.jv64_off = al(2 * v64);
-    size_t lg = 0;                                 // float pairs
-    for (int k = 0; k < L; ++k)
-      lg = std::max(lg, jacobi_reg_log_sweep(imin(imin(j.qb[k], 2 * imin(j.chi, j.qb[k + 1])), 128)));
-    j.lay.log_off = al(2 * lg * JR_LOG_SWEEPS);
   } else {
     j.lay.jw64_off = j.lay.jv64_off = 0;
+  }
+  if (j.refine) {
+    size_t lg = 0, j32 = 0, vb = 0;                // float pairs, floats, doubles
+    for (int k = 0; k < L; ++k) {
+      const int ncol = imin(j.qb[k], 2 * imin(j.chi, j.qb[k + 1]));
+      lg = std::max(lg, jacobi_reg_log_sweep(imin(ncol, 128)));
+      j32 = std::max(j32, (size_t)ncol * jacobi_ld<float>(ncol));
+      vb = std::max(vb, (size_t)ncol * jacobi_ld<double>(ncol) + ncol);
+    }
+    const size_t fpe = eb / 4;                     // floats per element
+    j.lay.log_off = al(2 * lg * JR_LOG_SWEEPS / fpe);
+    j.lay.j32_off = al((j32 + fpe - 1) / fpe);
+    j.lay.vb64_off = al((2 * vb + CL_MAX * 8) / fpe);
   }
   j.lay.total = off;
 }
@@ -594,7 +605,7 @@ template <typename S>
 __device__ inline void stage_rows(const S* V, int ld, int ncol, int k0, int nk, int kc, double* st) {
   for (int idx = threadIdx.x; idx < ncol * nk; idx += blockDim.x) {
     const int c = idx / nk, kk = idx - c * nk;
-    st[(size_t)c * kc + kk] = (double)__ldcg(V + (size_t)c * ld + k0 + kk);
+    st[(size_t)c * kc + kk] = rf_d(__ldcg(V + (size_t)c * ld + k0 + kk));
   }
 }
 
@@ -661,9 +672,9 @@ __device__ inline void rows_ns_step(const RowsLayout& R, unsigned char* wa, cons
 // Jacobi runs on the columns of C^T) for the rows [i0, i0 + li), read from
 // the job's scratch, and V (ncol x ncol, FP64, column c at V + c * ld), both
 // staged in chunks of kc indices k.
-template <typename T>
+template <typename T, typename N>
 __device__ inline void rows_xv(const RowsLayout& R, unsigned char* wa, const T* C, int n, bool trans, double scl,
-                               int i0, int li, const double* V, int ld, double* W, int ncol) {
+                               int i0, int li, const N* V, int ld, double* W, int ncol) {
   double* st = (double*)(wa + R.st);
   double* xs = (double*)(wa + R.xs);                      // xs[kk * li + ii] = X(i0 + ii, k0 + kk)
   const int kc = R.kc;
@@ -671,7 +682,7 @@ __device__ inline void rows_xv(const RowsLayout& R, unsigned char* wa, const T* 
   for (int k0 = 0; k0 < ncol; k0 += kc) {
     const int nk = imin(kc, ncol - k0);
     __syncthreads();
-    stage_rows<double>(V, ld, ncol, k0, nk, kc, st);
+    stage_rows<N>(V, ld, ncol, k0, nk, kc, st);
     for (int idx = threadIdx.x; idx < nk * li; idx += blockDim.x) {
       const int kk = idx / li, ii = idx - kk * li, i = i0 + ii, k = k0 + kk;
       xs[idx] = scl * (double)__ldcg(trans ? C + (size_t)i * n + k : C + (size_t)k * n + i);
@@ -700,17 +711,18 @@ __device__ inline void rows_xv(const RowsLayout& R, unsigned char* wa, const T* 
 // [c len / P, (c+1) len / P) of every column of W and [c ncol / P,
 // (c+1) ncol / P) of every column of V.  Every CTA sums the exchanged parts
 // in the same order, so every CTA takes the same rotations.
-// FP32 data (T = float): the leader has already run FP32 sweeps on X alone and
-// logged their rotations (sw32 sweeps; every CTA forms its rows of their product
-// V0 from the log), or, with sw32 < 0, left V0 (FP32, ncol x ncol) in the job's
-// scratch; one FP64
-// Newton-Schulz step, spread over the CTAs by blocks of columns, makes it
-// orthogonal to FP64 working accuracy (V0^T V0 - I ~ 1e-6 becomes ~1e-12),
-// W = X V is formed in FP64 and the FP64 sweeps start from there -- the
-// result is an FP64 one-sided Jacobi SVD of X started from the FP32 sweeps'
-// V.  FP64 data start from W = X, V = I.  Column norms are recomputed
-// exactly at the start of every sweep and at the end.  Every CTA then finds
-// the same singular values, order and kept rank (the rank rule of Eq.
+// The start, by sw32:
+// >= 0: the leader has run FP32 sweeps on X alone and logged their rotations; every
+//   CTA forms its rows of their product V0 from the log, and rf_refine takes V0 to an
+//   orthonormal V with W = X V and orthogonal columns, to 48 (FP32 data) or 53 bits;
+//   the FP64 sweeps run only where it could not finish, from the V it reached;
+// -1 (FP32 data beyond the register Jacobi): the leader's V0 is in the job's scratch;
+//   one FP64 Newton-Schulz step, spread over the CTAs by blocks of columns, makes it
+//   orthogonal to ~1e-12, W = X V is formed in FP64 and the FP64 sweeps finish;
+// -2, and FP64 data: FP64 sweeps from W = X, V = I.
+// Column norms are recomputed exactly at the start of every sweep and at the end.
+// Every CTA then finds the same singular values, order and kept rank (the rank rule
+// of Eq.
 // svd-move with delta) and writes its rows of core k (V^T[:r], r x n) and of
 // U S (m x r).  Called by all threads of every CTA with equal arguments;
 // returns the kept rank (0 if it exceeds the bond capacity), the FP64
@@ -740,17 +752,78 @@ __device__ int svd64_rows(ClusterCtx& cc, const RoundJob& J, int L, int k, int m
   const int i0 = cc.rank * len / cc.P, li = (cc.rank + 1) * len / cc.P - i0;
   const int v0 = cc.rank * ncol / cc.P, vi = (cc.rank + 1) * ncol / cc.P - v0;
   double* W = Wl;
-  if constexpr (two_phase) {
+  const double tol64 = 16.0 * 2.220446049250313e-16 * sqrt((double)len);
+  auto xat = [&](int i, int kk) -> double { return scl * (double)__ldcg(trans ? C + (size_t)i * n + kk : C + (size_t)kk * n + i); };
+  const int ld1 = jacobi_ld<double>(ncol);
+  int state = RF_SWEEPS;
+  if (sw32 >= 0) {
+    // start from the leader's logged FP32 sweeps, refine by products
+    const long long t0 = clock64();
+    using N = typename std::conditional<two_phase, float2, double>::type;
+    RefineMem<N> rm;
+    rm.V = (N*)(scr + J.lay.jv64_off);
+    rm.stat = (float*)(scr + J.lay.vb64_off);     // 16-byte aligned, then V2 and the norms
+    rm.V2 = (N*)(rm.stat + CL_MAX * 8);
+    rm.W = (N*)(scr + J.lay.jw64_off);
+    rm.J = (float*)(scr + J.lay.j32_off);
+    rm.ldv = ld1;
+    rm.ldw = jacobi_ld<double>(len);
+    rm.ldj = jacobi_ld<float>(ncol);
+    rm.nrm = rm.V2 + (size_t)ncol * ld1;
+    rm.log = (float2*)(scr + J.lay.log_off);
+    jacobi_reg_apply(rm.log, sw32, ncol, v0, vi, rm.V, ld1, (float2*)wa);
+    cl_sync(cc);
+    // one more FP32 Jacobi, of W: the leader's sweeps, their product over the cluster
+    auto jacobi = [&]() -> bool {
+      int sw = 0;
+      if (cc.rank == 0) {
+        float* Wf = (float*)wa;
+        const int ldw32 = jacobi_reg_ld(len), ncp = jacobi_reg_cols(ncol);
+        for (int idx = threadIdx.x; idx < ncp * ldw32; idx += blockDim.x) {
+          const int jj = idx / ldw32, i = idx % ldw32;
+          // 2^20: columns down to 1e-18 of the scale are above the Jacobi's floor
+          Wf[idx] = jj < ncol && i < len ? 1048576.f * rf_f(__ldcg(rm.W + (size_t)jj * rm.ldw + i)) : 0.f;
+        }
+        __syncthreads();
+        sw = jacobi_reg<true>(Wf, ncol, len, imin(maxsw, JR_LOG_SWEEPS), rm.log);
+        if (cl_alive(cc) && threadIdx.x < (unsigned)cc.P) cl_store_remote(&cc.sh->cmd.sw32, threadIdx.x, sw);
+      }
+      if (!cl_sync(cc)) return false;
+      sw = *(volatile int*)&cc.sh->cmd.sw32;
+      __syncthreads();
+      jacobi_reg_apply(rm.log, sw, ncol, v0, vi, rm.J, rm.ldj, (float2*)wa);
+      return cl_sync(cc);
+    };
+    const T tscl = (T)scl;                        // exact: a power of two
+    auto xn = [&](int i, int kk) -> N { return rf_make<N>(tscl * __ldcg(trans ? C + (size_t)i * n + kk : C + (size_t)kk * n + i)); };
+    // the sums of FP32 data carry 48 bits
+    const float tol2r = (two_phase ? 256.f : 1.f) * (float)(tol64 * tol64);
+    state = rf_refine<N>(cc, rm, ncol, len, sw32 < maxsw, xn, trans, trans, tol2r,
+                         two_phase ? 2e-13f : 2e-15f, two_phase ? 2e-6f : 2e-9f, two_phase ? 1e-11f : 1e-14f,
+                         two_phase ? 1e-22f : 1e-27f, SM_SMALL, SM_WORK, jacobi);
+    if (phase_acc && threadIdx.x == 0) phase_acc[PH_NS] += (double)(clock64() - t0);
+    const long long t1 = clock64();
+    for (int idx = threadIdx.x; idx < ncol * vi; idx += blockDim.x) {
+      const int j = idx / vi, ii = idx % vi;
+      Vl[(size_t)j * R.lv + ii] = rf_d(__ldcg(rm.V + (size_t)j * ld1 + v0 + ii));
+    }
+    if (state == RF_DONE) {
+      for (int idx = threadIdx.x; idx < ncol * li; idx += blockDim.x) {
+        const int j = idx / li, ii = idx % li;
+        Wl[(size_t)j * R.lw + ii] = rf_d(__ldcg(rm.W + (size_t)j * rm.ldw + i0 + ii));
+      }
+      __syncthreads();
+    } else {
+      rows_xv(R, wa, C, n, trans, scl, i0, li, rm.V, ld1, W, ncol);
+    }
+    cl_sync(cc);                                  // the staging space is the exchange buffers' again
+    if (phase_acc && threadIdx.x == 0) phase_acc[PH_XV] += (double)(clock64() - t1);
+  } else if (two_phase && sw32 == -1) {
     const long long t0 = clock64();
     float* V0 = (float*)(scr + J.lay.jv_off);
-    const int ld0 = jacobi_ld<float>(ncol), ld1 = jacobi_ld<double>(ncol);
-    if (sw32 >= 0) {
-      // this CTA's rows of V0 from the leader's log
-      jacobi_reg_apply((const float2*)(scr + J.lay.log_off), sw32, ncol, v0, vi, V0, ld0, (float2*)wa);
-      cl_sync(cc);
-    }
+    const int ld0 = jacobi_ld<float>(ncol);
     double* V1 = (double*)(scr + J.lay.jv64_off);
-    rows_ns_step<float>(R, wa, V0, ld0, V1, ld1, ncol, v0, vi);
+    rows_ns_step(R, wa, V0, ld0, V1, ld1, ncol, v0, vi);
     cl_sync(cc);                                  // every block of V1 written (cluster-scope fence)
     if (phase_acc && threadIdx.x == 0) phase_acc[PH_NS] += (double)(clock64() - t0);
     const long long t1 = clock64();
@@ -758,15 +831,14 @@ __device__ int svd64_rows(ClusterCtx& cc, const RoundJob& J, int L, int k, int m
       const int j = idx / vi, ii = idx % vi;
       Vl[(size_t)j * R.lv + ii] = __ldcg(V1 + (size_t)j * ld1 + v0 + ii);
     }
-    rows_xv<T>(R, wa, C, n, trans, scl, i0, li, V1, ld1, W, ncol);
+    rows_xv(R, wa, C, n, trans, scl, i0, li, V1, ld1, W, ncol);
     cl_sync(cc);                                  // the staging space is the exchange buffers' again
     if (phase_acc && threadIdx.x == 0) phase_acc[PH_XV] += (double)(clock64() - t1);
   } else {
     // own rows of X (promoted, scaled by a power of two: exact)
     for (int idx = threadIdx.x; idx < ncol * li; idx += blockDim.x) {
-      const int j = idx / li, ii = idx % li, i = i0 + ii;
-      const T v = trans ? __ldcg(C + (size_t)i * n + j) : __ldcg(C + (size_t)j * n + i);
-      Wl[(size_t)j * R.lw + ii] = scl * (double)v;
+      const int j = idx / li, ii = idx % li;
+      Wl[(size_t)j * R.lw + ii] = xat(i0 + ii, j);
     }
     for (int idx = threadIdx.x; idx < ncol * vi; idx += blockDim.x) {
       const int j = idx / vi, ii = idx % vi;
@@ -774,11 +846,10 @@ __device__ int svd64_rows(ClusterCtx& cc, const RoundJob& J, int L, int k, int m
     }
     __syncthreads();
   }
-  const double tol64 = 16.0 * 2.220446049250313e-16 * sqrt((double)len);
-  bool conv = false;
-  int rounds = 0;
-  const int sw = rows_sweeps<double>(cc, R, wa, W, Vl, ncol, li, vi, maxsw, tol64 * tol64, &s_nrot, phase_acc,
-                                     &conv, &rounds);
+  bool conv = state == RF_DONE;
+  int rounds = 0, sw = 0;
+  if (state != RF_DONE)
+    sw = rows_sweeps<double>(cc, R, wa, W, Vl, ncol, li, vi, maxsw, tol64 * tol64, &s_nrot, phase_acc, &conv, &rounds);
   *sweeps_out = sw;
   *noconv = !conv || cc.dead;
   if (exec_flops && threadIdx.x == 0) {
@@ -906,13 +977,14 @@ __device__ __noinline__ int svd64_site(const RoundJob& J, int L, int k, const T*
     pc.lap(PH_SVD_OUT);
     int sw32 = 0;
     bool logged = false;
-    if constexpr (sizeof(T) == 4) {
-      // FP32 data: FP32 sweeps on X by this CTA alone (its own stopping rule, a
+    const bool plain = ncol < RF_MIN;             // FP64 sweeps from V = I
+    if (!plain && (sizeof(T) == 4 || J.refine)) {
+      // FP32 sweeps on X by this CTA alone (its own stopping rule, a
       // sweep limit, convergence not required).  In registers where X fits: W only,
       // the rotations logged for the cluster to form V0 (a row of V0 per half-warp,
       // ~1/16 of the sweeps' time on 16 CTAs, where carrying V along would double
       // the sweeps' work)
-      if (jacobi_reg_fits(ncol, len)) {
+      if (J.refine && jacobi_reg_fits(ncol, len) && rf_bytes(ncol, len, cc.P) <= (size_t)SM_WORK) {
         float* Wf = (float*)work;
         const int ldw32 = jacobi_reg_ld(len), ncp = jacobi_reg_cols(ncol);
         for (int idx = threadIdx.x; idx < ncp * ldw32; idx += blockDim.x) {
@@ -924,7 +996,7 @@ __device__ __noinline__ int svd64_site(const RoundJob& J, int L, int k, const T*
         sw32 = jacobi_reg<true>(Wf, ncol, len, imin(maxsw, JR_LOG_SWEEPS), (float2*)(scr + J.lay.log_off));
         logged = true;
         __threadfence();                          // the log, before the workers are told of it
-      } else {
+      } else if constexpr (sizeof(T) == 4) {
         // larger: the in-CTA Jacobi of the FP32 path, V0 left in the job's scratch
         const int ldw32 = jacobi_ld<float>(len), ldv32 = jacobi_ld<float>(ncol);
         const size_t need32 = ((size_t)ncol * ldw32 + (size_t)ncol * ldv32) * sizeof(float);
@@ -947,11 +1019,11 @@ __device__ __noinline__ int svd64_site(const RoundJob& J, int L, int k, const T*
       if (threadIdx.x == 0) pc.acc[PH_SWEEPS32] += sw32;
       pc.lap(PH_J32);
     }
-    cl_command(cc, 2, ncol, len, maxsw, m, n, k, delta, scl, logged ? sw32 : -1);
+    cl_command(cc, 2, ncol, len, maxsw, m, n, k, delta, scl, logged ? sw32 : plain ? -2 : -1);
     int sw = 0;
     bool noconv = false;
     double xfl = 0.0;
-    const int r = svd64_rows<T>(cc, J, L, k, m, n, scl, delta, maxsw, logged ? sw32 : -1, &sw, &noconv, &xfl,
+    const int r = svd64_rows<T>(cc, J, L, k, m, n, scl, delta, maxsw, logged ? sw32 : plain ? -2 : -1, &sw, &noconv, &xfl,
                                 pc.on ? pc.acc : nullptr);
     pc.lap(PH_JACOBI);
     if (threadIdx.x == 0) { pc.acc[PH_SVD64_FLOPS] += svd_flops(m, n); pc.acc[PH_SVD64_EXEC] += xfl; }
