@@ -1248,10 +1248,10 @@ static int macro_impl(tnlbm_sim* s, double* rho, double* u) {
     return fin(TNLBM_E_OOM);
   }
   double *dr = d, *jx = d + nc, *jy = d + 2 * nc, *jz = d + 3 * nc;
-  for (int i = 0; i < s->lat.Q; ++i) {
-    contract_dense_f64<T>(s->nodes[s->f_state[i]], s->n, tmp, scr, sb, s->s0);
-    launch_accum_moments<double>(tmp, nc, dr, jx, jy, jz, s->lat.c[i][0], s->lat.c[i][1], s->lat.c[i][2], i == 0, s->s0);
-  }
+  contract_begin(scr, s->s0);
+  for (int i = 0; i < s->lat.Q; ++i)
+    contract_moments<T>(s->nodes[s->f_state[i]], s->n, tmp, scr, sb, dr, jx, jy, jz, s->lat.c[i][0], s->lat.c[i][1],
+                        s->lat.c[i][2], i == 0, s->s0);
   if (s->mask_node >= 0) {
     if (cudaMalloc(&dm, nc * sizeof(double)) != cudaSuccess) return fin(TNLBM_E_OOM);
     contract_dense_f64<T>(s->nodes[s->mask_node], s->n, dm, scr, sb, s->s0);
@@ -1259,9 +1259,7 @@ static int macro_impl(tnlbm_sim* s, double* rho, double* u) {
   if (u) launch_velocity(nc, dr, jx, jy, jz, dm, s->cfg.force[0], s->cfg.force[1], s->cfg.force[2], s->s0);
   if (rho) cudaMemcpyAsync(rho, dr, nc * sizeof(double), cudaMemcpyDeviceToHost, s->s0);
   if (u) cudaMemcpyAsync(u, jx, 3 * nc * sizeof(double), cudaMemcpyDeviceToHost, s->s0);
-  cudaError_t e = cudaStreamSynchronize(s->s0);
-  if (e != cudaSuccess) return fin(cuda_fail(e, "tnlbm_macroscopic"));
-  return fin(0);
+  return fin(contract_end(scr, s->s0, "tnlbm_macroscopic"));
 }
 
 template <typename T>
@@ -1845,12 +1843,11 @@ int tnlbm_to_dense(int precision, int n_bits, const void* X, const int* rX, int 
   const size_t sb = tn::contract_scratch_bytes(n_bits, capX, es);
   tn::DevBuf scr;
   if (!scr.alloc(sb)) { set_error("out of device memory"); return TNLBM_E_OOM; }
+  tn::contract_begin(scr.p, st);
   int rc = precision == TNLBM_FP64 ? tn::contract_dense<double>(m, n_bits, (double*)dense, scr.p, sb, st)
                                    : tn::contract_dense<float>(m, n_bits, (float*)dense, scr.p, sb, st);
   if (rc) return rc;
-  TN_CUDA(cudaGetLastError());
-  TN_CUDA(cudaStreamSynchronize(st));
-  return 0;
+  return tn::contract_end(scr.p, st, "tnlbm_to_dense");
 }
 
 int tnlbm_from_dense(int precision, int n_bits, const void* dense, void* dst, int* dst_ranks, int dst_cap,

@@ -98,19 +98,40 @@ void launch_mass_fix(const MpsRef* d_refs, int n, int L, double* d_mass, const d
 template <typename T>
 void launch_copy(const MpsRef* d_src, const MpsRef* d_dst, int n, int L, cudaStream_t st);
 
+// site-ordered linear index of cell (x, y, z): site k (MSB first) holds bit
+// (n-1-k/3) of coordinate k%3
+__host__ __device__ inline size_t site_index(int x, int y, int z, int n) {
+  size_t idx = 0;
+  const int c[3] = {x, y, z};
+  for (int k = 0; k < 3 * n; ++k) idx = (idx << 1) | (size_t)((c[k % 3] >> (n - 1 - k / 3)) & 1);
+  return idx;
+}
+
+// ---- contract.cu
+// The scratch of a contraction starts with a status word: contract_begin clears it,
+// contract_end waits for the stream and reports it (one pair may span several
+// contractions on the stream).
+void contract_begin(void* d_scratch, cudaStream_t st);
+int contract_end(const void* d_scratch, cudaStream_t st, const char* what);
 // dense[x][y][z] = contraction of X (host-known ranks not needed)
 template <typename T>
 int contract_dense(const MpsRef& X, int n_bits, T* d_dense, void* d_scratch, size_t scratch_bytes,
                    cudaStream_t st);
 size_t contract_scratch_bytes(int n_bits, int cap, size_t elem);
+template <typename T>
+int contract_dense_f64(const MpsRef& X, int n_bits, double* d_dense, void* d_scratch, size_t scratch_bytes,
+                       cudaStream_t st);
+// rho (+)= f, j (+)= c f for the field f of X (tmp: a field of free space)
+template <typename T>
+int contract_moments(const MpsRef& X, int n_bits, double* tmp, void* d_scratch, size_t scratch_bytes, double* rho,
+                     double* jx, double* jy, double* jz, int cx, int cy, int cz, int first, cudaStream_t st);
+
+// ---- misc.cu
 // plane coordinate[axis] = index of X, out[u * N + v] (the two other axes in order)
 size_t plane_scratch_bytes(int n_bits, int axis, int cap);
 template <typename T>
 int contract_plane_f64(const MpsRef& X, int n_bits, int axis, int index, double* d_plane, void* d_scratch,
                        size_t scratch_bytes, cudaStream_t st);
-template <typename T>
-int contract_dense_f64(const MpsRef& X, int n_bits, double* d_dense, void* d_scratch, size_t scratch_bytes,
-                       cudaStream_t st);
 
 // accumulate rho += f, j += c f (double) from a dense population
 template <typename T>

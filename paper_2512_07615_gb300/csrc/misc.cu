@@ -1,7 +1,7 @@
 // Smaller kernels of the MPS-LBM step and of the library's input/output:
 //  - <X, 1>: transfer-vector sweep (Sec. 3.2, mean density rho_0)
 //  - rho_0 and the scalar coefficients of the Taylor 1/rho (Sec. 3.2)
-//  - contraction of an MPS to a dense [x][y][z] field (Eq. MPS), for outputs
+//  - planes of an MPS, for outputs
 //  - moments and velocity of the contracted populations (Eq. macro, App. A)
 //  - TT-SVD of a dense field (Eq. svd-comp), used to compress geometry masks
 #include <algorithm>
@@ -108,115 +108,6 @@ __global__ void copy_kernel(const MpsRef* src, const MpsRef* dst, int L) {
 template <typename T>
 void launch_copy(const MpsRef* d_src, const MpsRef* d_dst, int n, int L, cudaStream_t st) {
   if (n > 0) copy_kernel<T><<<n, 256, 0, st>>>(d_src, d_dst, L);
-}
-
-// ---------------------------------------------------------------- dense contraction
-// site-ordered linear index of cell (x, y, z): site k (MSB first) holds bit
-// (n-1-k/3) of coordinate k%3
-__host__ __device__ inline size_t site_index(int x, int y, int z, int n) {
-  size_t idx = 0;
-  const int c[3] = {x, y, z};
-  for (int k = 0; k < 3 * n; ++k) idx = (idx << 1) | (size_t)((c[k % 3] >> (n - 1 - k / 3)) & 1);
-  return idx;
-}
-
-// Output contractions accumulate in FP64 whatever the storage type: they run
-// once per output, not on the hot path, and FP32 products of L cores would
-// bias sums over the lattice at the 1e-6 level.
-template <typename T>
-__global__ void left_rows_kernel(MpsRef X, int L, int h, double* Lm, int ldl) {
-  __shared__ double v[1024], w[1024];
-  const size_t l = blockIdx.x;
-  for (int k = 0; k < h; ++k) {
-    const int s = (int)((l >> (h - 1 - k)) & 1);
-    const int r0 = X.ranks[k], r1 = X.ranks[k + 1];
-    const T* A = (const T*)X.base + core_offset(L, X.cap, k);
-    for (int j = threadIdx.x; j < r1; j += blockDim.x) {
-      double acc = 0.0;
-      if (k == 0) acc = (double)A[(size_t)s * r1 + j];
-      else for (int i = 0; i < r0; ++i) acc += v[i] * (double)A[((size_t)i * 2 + s) * r1 + j];
-      w[j] = acc;
-    }
-    __syncthreads();
-    for (int j = threadIdx.x; j < r1; j += blockDim.x) v[j] = w[j];
-    __syncthreads();
-  }
-  const int rh = X.ranks[h];
-  for (int j = threadIdx.x; j < rh; j += blockDim.x) Lm[l * ldl + j] = v[j];
-}
-
-template <typename T>
-__global__ void right_cols_kernel(MpsRef X, int L, int h, double* Rt, int ldr) {
-  __shared__ double v[1024], w[1024];
-  const size_t q = blockIdx.x;
-  for (int k = L - 1; k >= h; --k) {
-    const int s = (int)((q >> (L - 1 - k)) & 1);
-    const int r0 = X.ranks[k], r1 = X.ranks[k + 1];
-    const T* A = (const T*)X.base + core_offset(L, X.cap, k);
-    for (int i = threadIdx.x; i < r0; i += blockDim.x) {
-      double acc = 0.0;
-      if (k == L - 1) acc = (double)A[(size_t)i * 2 + s];
-      else for (int j = 0; j < r1; ++j) acc += (double)A[((size_t)i * 2 + s) * r1 + j] * v[j];
-      w[i] = acc;
-    }
-    __syncthreads();
-    for (int i = threadIdx.x; i < r0; i += blockDim.x) v[i] = w[i];
-    __syncthreads();
-  }
-  const int rh = X.ranks[h];
-  for (int j = threadIdx.x; j < rh; j += blockDim.x) Rt[q * ldr + j] = v[j];
-}
-
-template <typename T>
-__global__ void join_kernel(MpsRef X, int n, int h, const double* Lm, const double* Rt, int ld, T* out) {
-  const int L = 3 * n;
-  const size_t N = (size_t)1 << n;
-  const size_t total = N * N * N;
-  const int rh = X.ranks[h];
-  for (size_t idx = blockIdx.x * (size_t)blockDim.x + threadIdx.x; idx < total;
-       idx += (size_t)gridDim.x * blockDim.x) {
-    const int z = (int)(idx % N), y = (int)((idx / N) % N), x = (int)(idx / (N * N));
-    const size_t si = site_index(x, y, z, n);
-    const size_t l = si >> (L - h), q = si & (((size_t)1 << (L - h)) - 1);
-    const double* a = Lm + l * ld;
-    const double* b = Rt + q * ld;
-    double acc = 0.0;
-    for (int j = 0; j < rh; ++j) acc += a[j] * b[j];
-    out[idx] = (T)acc;
-  }
-}
-
-size_t contract_scratch_bytes(int n_bits, int cap, size_t elem) {
-  const int L = 3 * n_bits, h = L / 2;
-  const size_t ld = bond_cap(L, cap, h);
-  (void)elem;
-  return (((size_t)1 << h) + ((size_t)1 << (L - h))) * ld * sizeof(double);
-}
-
-template <typename T, typename OutT>
-int contract_dense_to(const MpsRef& X, int n_bits, OutT* d_dense, void* d_scratch, size_t scratch_bytes,
-                      cudaStream_t st) {
-  const int L = 3 * n_bits, h = L / 2;
-  const int ld = bond_cap(L, X.cap, h);
-  if (contract_scratch_bytes(n_bits, X.cap, sizeof(T)) > scratch_bytes) return TNLBM_E_ARG;
-  double* Lm = (double*)d_scratch;
-  double* Rt = Lm + ((size_t)1 << h) * ld;
-  left_rows_kernel<T><<<(unsigned)(1u << h), 256, 0, st>>>(X, L, h, Lm, ld);
-  right_cols_kernel<T><<<(unsigned)(1u << (L - h)), 256, 0, st>>>(X, L, h, Rt, ld);
-  join_kernel<OutT><<<152 * 16, 256, 0, st>>>(X, n_bits, h, Lm, Rt, ld, d_dense);
-  return 0;
-}
-
-template <typename T>
-int contract_dense(const MpsRef& X, int n_bits, T* d_dense, void* d_scratch, size_t scratch_bytes,
-                   cudaStream_t st) {
-  return contract_dense_to<T, T>(X, n_bits, d_dense, d_scratch, scratch_bytes, st);
-}
-
-template <typename T>
-int contract_dense_f64(const MpsRef& X, int n_bits, double* d_dense, void* d_scratch, size_t scratch_bytes,
-                       cudaStream_t st) {
-  return contract_dense_to<T, double>(X, n_bits, d_dense, d_scratch, scratch_bytes, st);
 }
 
 // ---------------------------------------------------------------- plane contraction
@@ -586,8 +477,6 @@ int tt_svd_dense(const T* d_dense, int n, T* d_dst, int* d_dst_ranks, int dst_ca
   template void launch_rho0<T>(const MpsRef*, int, double, double*, cudaStream_t);              \
   template void launch_copy<T>(const MpsRef*, const MpsRef*, int, int, cudaStream_t);           \
   template void launch_mass_fix<T>(const MpsRef*, int, int, double*, const double*, cudaStream_t); \
-  template int contract_dense<T>(const MpsRef&, int, T*, void*, size_t, cudaStream_t);          \
-  template int contract_dense_f64<T>(const MpsRef&, int, double*, void*, size_t, cudaStream_t);  \
   template void launch_accum_moments<T>(const T*, size_t, double*, double*, double*, double*,   \
                                         int, int, int, int, cudaStream_t);                       \
   template int tt_svd_dense<T>(const T*, int, T*, int*, int, int, double, int*, cudaStream_t); \
