@@ -54,79 +54,6 @@ __device__ inline double block_sum(double v, double* red) {
   return s;
 }
 
-// One-sided Jacobi on ncol columns of length len, stored column-contiguous
-// (Wm[j*len + i]); V (ncol x ncol, V[j*ncol + i] = column j) accumulates the
-// rotations.  Parallel ordering: a round-robin tournament, one warp per pair.
-// Returns the number of sweeps used (maxsw + 1 if not converged).
-template <typename T>
-__device__ int jacobi_cols(T* Wm, T* V, int ncol, int len, int maxsw) {
-  for (int idx = threadIdx.x; idx < ncol * ncol; idx += blockDim.x)
-    V[idx] = (idx / ncol == idx % ncol) ? (T)1 : (T)0;
-  __shared__ int s_rot;
-  __syncthreads();
-  if (ncol < 2) return 0;
-  const int np = (ncol + 1) & ~1;          // padded to even; index np-1 may be a dummy
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
-  // stopping threshold on |cos| of a pair: a few ulps above the round-off of a
-  // freshly rotated pair, so short columns cannot cycle on noise
-  const double tol = 16.0 * Eps<T>::v * sqrt((double)len);
-  int sweep = 0;
-  for (; sweep < maxsw; ++sweep) {
-    if (threadIdx.x == 0) s_rot = 0;
-    __syncthreads();
-    for (int rnd = 0; rnd < np - 1; ++rnd) {
-      for (int p = wid; p < np / 2; p += nw) {
-        int a, b;
-        if (p == 0) { a = rnd; b = np - 1; }
-        else { a = (rnd + p) % (np - 1); b = (rnd - p + (np - 1)) % (np - 1); }
-        if (a >= ncol || b >= ncol) continue;
-        if (a > b) { int t = a; a = b; b = t; }
-        T* wa = Wm + (size_t)a * len;
-        T* wb = Wm + (size_t)b * len;
-        double al = 0, be = 0, ga = 0;
-        for (int i = lane; i < len; i += 32) {
-          double x = (double)wa[i], y = (double)wb[i];
-          al += x * x; be += y * y; ga += x * y;
-        }
-        for (int o = 16; o > 0; o >>= 1) {
-          al += __shfl_xor_sync(0xffffffffu, al, o);
-          be += __shfl_xor_sync(0xffffffffu, be, o);
-          ga += __shfl_xor_sync(0xffffffffu, ga, o);
-        }
-        // pairs below the representable range carry nothing; skip them too
-        if (ga == 0.0 || al < 1e-250 || be < 1e-250 || fabs(ga) <= tol * sqrt(al) * sqrt(be)) continue;
-        // Rutishauser's rotation zeroing the (a, b) inner product
-        double zeta = (be - al) / (2.0 * ga);
-        double t = (zeta >= 0 ? 1.0 : -1.0) / (fabs(zeta) + sqrt(1.0 + zeta * zeta));
-        double c = 1.0 / sqrt(1.0 + t * t), s = c * t;
-        const T cc = (T)c, ss = (T)s;
-        for (int i = lane; i < len; i += 32) {
-          T x = wa[i], y = wb[i];
-          wa[i] = cc * x - ss * y;
-          wb[i] = ss * x + cc * y;
-        }
-        T* va = V + (size_t)a * ncol;
-        T* vb = V + (size_t)b * ncol;
-        for (int i = lane; i < ncol; i += 32) {
-          T x = va[i], y = vb[i];
-          va[i] = cc * x - ss * y;
-          vb[i] = ss * x + cc * y;
-        }
-        if (lane == 0) s_rot = 1;
-      }
-      __syncthreads();
-    }
-    int any = s_rot;
-    __syncthreads();
-    if (!any) break;
-  }
-  return sweep;
-}
-
-}  // namespace tn
-
-namespace tn {
-
 // ---------------------------------------------------------------- fast in-CTA kernels
 // Designed for 1024-thread CTAs with the working matrix in shared memory.
 
@@ -344,7 +271,8 @@ __device__ void householder_qr_par(T* A, int m, int n, int lda, T* Q, int ldq, T
   __syncthreads();
 }
 
-// One-sided Jacobi as jacobi_cols, with a half-warp per column pair so that a
+// One-sided Jacobi (a round-robin tournament of pairs, V accumulating the rotations)
+// on columns stored contiguously, with a half-warp per column pair so that a
 // 1024-thread CTA keeps 64 pairs in flight.  Columns have stride ldw >= len.
 template <typename T>
 __device__ int jacobi_cols_hw(T* Wm, int ldw, T* V, int ldv, int ncol, int len, int maxsw) {

@@ -303,59 +303,6 @@ __global__ void gram_reduce_kernel(const double* part, int P, size_t mm, double*
   }
 }
 
-// eigen-decomposition of the symmetric PSD Gram G (m x m) by one-sided Jacobi;
-// truncation; writes U (m x r, FP64) and the rank.
-__global__ void __launch_bounds__(1024) gram_eig_kernel(double* G, int m, double* Wm, double* Vm,
-                                                        double* U, int chi, double delta2,
-                                                        int ncols_cap, int* r_out, int* status) {
-  __shared__ double lam[1024];
-  __shared__ int perm[1024];
-  for (int e = threadIdx.x; e < m * m; e += blockDim.x) {
-    const int i = e / m, j = e % m;
-    const double v = (j >= i) ? G[(size_t)i * m + j] : G[(size_t)j * m + i];
-    Wm[(size_t)j * m + i] = v;   // column j
-  }
-  __syncthreads();
-  int sw = jacobi_cols<double>(Wm, Vm, m, m, 80);
-  if (sw >= 80 && threadIdx.x == 0) atomicOr(status, ST_NOCONV);
-  for (int j = threadIdx.x; j < m; j += blockDim.x) {
-    double a = 0.0;
-    for (int i = 0; i < m; ++i) a += Wm[(size_t)j * m + i] * Wm[(size_t)j * m + i];
-    const double lj = sqrt(a);                // eigenvalue of G = sigma^2 of M
-    if (!(lj >= 0.0) || isinf(lj)) { lam[j] = -1.0; atomicOr(status, ST_NAN); }   // orders last
-    else lam[j] = lj;
-  }
-  __syncthreads();
-  for (int j = threadIdx.x; j < m; j += blockDim.x) {
-    int rank = 0;
-    for (int o = 0; o < m; ++o) rank += (lam[o] > lam[j]) || (lam[o] == lam[j] && o < j);
-    perm[rank] = j;
-  }
-  __syncthreads();
-  __shared__ int s_r;
-  if (threadIdx.x == 0) {
-    const int rmax = imin(chi, imin(m, ncols_cap));
-    int r = rmax;
-    // eigenvalues of the Gram matrix below its round-off level carry no
-    // information: treat that level as the smallest resolvable tail
-    const double floor2 = 64.0 * 2.220446049250313e-16 * (double)m * lam[perm[0]];
-    const double thr = delta2 > floor2 ? delta2 : floor2;
-    for (int rr = 1; rr <= rmax; ++rr) {
-      double tail = 0.0;
-      for (int p = rr; p < m; ++p) tail += lam[perm[p]];
-      if (tail <= thr) { r = rr; break; }
-    }
-    s_r = r;
-    *r_out = r;
-  }
-  __syncthreads();
-  const int r = s_r;
-  for (int e = threadIdx.x; e < m * r; e += blockDim.x) {
-    const int i = e / r, j = e % r;
-    U[e] = Vm[(size_t)perm[j] * m + i];
-  }
-}
-
 // Mn (r x ncols) = U^T (r x m) M (m x ncols)
 __global__ void project_kernel(const double* U, int m, int r, const double* M, size_t ncols, double* Mn) {
   const size_t total = (size_t)r * ncols;
@@ -408,27 +355,30 @@ int tt_svd_dense(const T* d_dense, int n, T* d_dst, int* d_dst_ranks, int dst_ca
   const size_t total = (size_t)1 << L;
   const int mmax = 2 * imin(chi_max, dst_cap);
   if (mmax > 1024) return TNLBM_E_ARG;
-  double *M = nullptr, *M2 = nullptr, *G = nullptr, *Wm = nullptr, *Vm = nullptr, *U = nullptr, *nrm = nullptr;
+  double *M = nullptr, *M2 = nullptr, *G = nullptr, *eig = nullptr, *U = nullptr, *nrm = nullptr;
   double* gpart = nullptr;
   int* d_r = nullptr;
+  RoundJob job, *d_job = nullptr;
+  const size_t eig_elems = plan_gram_eig(job, mmax);
   // partial Gram slices: as many as fit in 256 MB at the largest m (at most 304)
   const int NB_NORM = 152 * 4;
   int Pg = (int)std::min<size_t>(304, std::max<size_t>(1, ((size_t)256 << 20) / ((size_t)mmax * mmax * sizeof(double))));
   auto cleanup = [&]() {
-    cudaFree(M); cudaFree(M2); cudaFree(G); cudaFree(Wm); cudaFree(Vm); cudaFree(U); cudaFree(nrm); cudaFree(d_r);
+    cudaFree(M); cudaFree(M2); cudaFree(G); cudaFree(eig); cudaFree(d_job); cudaFree(U); cudaFree(nrm); cudaFree(d_r);
     cudaFree(gpart);
   };
   if (cudaMalloc(&M, total * sizeof(double)) != cudaSuccess ||
       cudaMalloc(&M2, total * sizeof(double)) != cudaSuccess ||
       cudaMalloc(&G, (size_t)mmax * mmax * sizeof(double)) != cudaSuccess ||
-      cudaMalloc(&Wm, (size_t)mmax * mmax * sizeof(double)) != cudaSuccess ||
-      cudaMalloc(&Vm, (size_t)mmax * mmax * sizeof(double)) != cudaSuccess ||
+      cudaMalloc(&eig, eig_elems * sizeof(double)) != cudaSuccess || cudaMalloc(&d_job, sizeof(RoundJob)) != cudaSuccess ||
       cudaMalloc(&U, (size_t)mmax * mmax * sizeof(double)) != cudaSuccess ||
       cudaMalloc(&nrm, NB_NORM * sizeof(double)) != cudaSuccess || cudaMalloc(&d_r, sizeof(int)) != cudaSuccess ||
       cudaMalloc(&gpart, (size_t)Pg * mmax * mmax * sizeof(double)) != cudaSuccess) {
     cleanup();
     return TNLBM_E_OOM;
   }
+  place_gram_eig(job, eig);
+  cudaMemcpyAsync(d_job, &job, sizeof(job), cudaMemcpyHostToDevice, st);
   to_site_order_kernel<T><<<152 * 8, 256, 0, st>>>(d_dense, n, M);
   norm2_part_kernel<<<NB_NORM, 256, 0, st>>>(M, total, nrm);
   std::vector<double> h_part(NB_NORM);
@@ -448,8 +398,8 @@ int tt_svd_dense(const T* d_dense, int n, T* d_dst, int* d_dst_ranks, int dst_ca
     const int P = (int)std::min<size_t>((size_t)Pg, nch);
     gram_part_kernel<<<P, 256, (size_t)m * kc * sizeof(double), st>>>(M, m, ncols, kc, P, gpart);
     gram_reduce_kernel<<<152, 256, 0, st>>>(gpart, P, (size_t)m * m, G);
-    gram_eig_kernel<<<1, 1024, 0, st>>>(G, m, Wm, Vm, U, imin(chi_max, dst_cap), delta * delta,
-                                        (int)(ncols < (size_t)1024 ? ncols : (size_t)1024), d_r, d_status);
+    launch_gram_eig(d_job, G, m, U, imin(chi_max, dst_cap), delta * delta,
+                    (int)(ncols < (size_t)1024 ? ncols : (size_t)1024), d_r, d_status, st);
     int h_r = 0;
     cudaMemcpyAsync(&h_r, d_r, sizeof(int), cudaMemcpyDeviceToHost, st);
     cudaError_t e = cudaStreamSynchronize(st);

@@ -1876,6 +1876,143 @@ __device__ void round_worker(const RoundJob& J, int L_arg, ClusterCtx& cc) {
   }
 }
 
+// ---------------------------------------------------------------- eigenvectors of a Gram matrix
+// The dominant eigenvectors U (m x r, row-major) of the symmetric positive
+// semi-definite G (m x m, its upper triangle) for the TT-SVD of a dense field, by
+// the centre SVD of the FP64 roundings (G = V diag V^T, V its right vectors) on one
+// cluster.  r: the smallest rank whose discarded eigenvalues sum to at most
+// max(delta2, the round-off level of the Gram matrix), capped at min(chi, m, ncols).
+//
+// A single CTA's FP64 Jacobi has two multiply-adds a clock: 25 k cycles a round of 48
+// pairs of 96, 10 ms a site.  The cluster's FP32 sweeps in registers and
+// refinement by products need ~0.3 ms.
+__global__ void __launch_bounds__(RT) gram_eig_kernel(const RoundJob* __restrict__ job, const double* __restrict__ G, int m,
+                                                      double* __restrict__ U, int chi, double delta2, int ncols_cap,
+                                                      int* r_out, int* status) {
+  __shared__ ClusterShared s_cl;
+  __shared__ double s_phase[PH_COUNT];
+  __shared__ double s_flops;
+  __shared__ int s_bad, s_rank;
+  extern __shared__ __align__(16) unsigned char smem[];
+  ClusterCtx cc;
+  const RoundJob& J = *job;
+  cl_init(cc, &s_cl, status, J.wait_ns > 0 ? J.wait_ns : 5000000000LL);
+  if (cc.rank == 0) {
+    double* scr = (double*)J.scratch;
+    double* C = scr + J.lay.c_off;
+    double* out = (double*)J.dst.base + core_offset(J.L, J.dst.cap, 1);
+    const SiteShared sh{(double*)(smem + SM_RED), (double*)(smem + SM_TAU), (double*)(smem + SM_SIG),
+                        (int*)smem, &s_bad, &s_rank, &s_flops};
+    PhaseClock pc(false, s_phase);
+    if (threadIdx.x == 0) { s_bad = 0; s_flops = 0.0; }
+    bool bad = false;
+    for (int e = threadIdx.x; e < m * m; e += blockDim.x) {
+      const int i = e / m, j = e % m;
+      const double v = j >= i ? G[e] : G[(size_t)j * m + i];
+      C[e] = v;
+      bad |= !isfinite(v);
+    }
+    bad = __syncthreads_or(bad);
+    // every non-zero singular value kept; the rank rule of the eigenvalues is below
+    const int kept = bad ? 0
+                         : svd64_site<double>(J, J.L, 1, C, m, m, out, scr + J.lay.us_off, scr,
+                                              (double*)(smem + SM_SMALL), sh, cc, status, nullptr, pc, 0.0);
+    if (bad && threadIdx.x == 0) flag(status, ST_NAN);
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      int r = 1;
+      if (kept > 0) {
+        const int rmax = imin(chi, imin(m, ncols_cap));
+        const double* lam = sh.sig;
+        const int* perm = sh.perm;
+        // eigenvalues below the Gram matrix's round-off level carry no information:
+        // that level is the smallest resolvable tail
+        const double floor2 = 64.0 * 2.220446049250313e-16 * (double)m * lam[perm[0]];
+        const double thr = delta2 > floor2 ? delta2 : floor2;
+        double tail = 0.0;
+        r = rmax;
+        for (int p = m - 1; p >= 1; --p) {
+          tail += lam[perm[p]];
+          if (!(tail <= thr)) break;
+          if (p <= rmax) r = p;
+        }
+      }
+      s_rank = r;
+      *r_out = r;
+    }
+    __syncthreads();
+    const int r = s_rank;
+    // (a zero singular value's vector is never within r unless G is zero)
+    for (int e = threadIdx.x; e < m * r; e += blockDim.x) {
+      const int i = e / r, j = e % r;
+      U[e] = j < kept ? out[(size_t)j * m + i] : (i == j ? 1.0 : 0.0);
+    }
+    cl_command(cc, 0, 0, 0, 0);
+  } else {
+    round_worker<double>(J, J.L, cc);
+  }
+  cl_exit(cc);
+}
+
+// Scratch of the eigenproblems of one TT-SVD (m <= mmax) as a job of one site.
+size_t plan_gram_eig(RoundJob& j, int mmax) {
+  j = RoundJob{};
+  j.L = 3;
+  j.n_bits = 1;
+  j.chi = mmax;
+  j.refine = 1;
+  j.dst.cap = mmax;
+  size_t off = 0;
+  auto al = [&](size_t n) { const size_t o = off; off += (n + 31) & ~(size_t)31; return o; };
+  const size_t ld = jacobi_ld<double>(mmax), n = mmax;
+  j.lay.c_off = al(n * n);
+  j.lay.us_off = al(n * n);
+  j.lay.jw64_off = j.lay.jw_off = al(n * ld);
+  j.lay.jv64_off = j.lay.jv_off = al(n * ld);
+  j.lay.log_off = al(jacobi_reg_log_sweep(imin(mmax, 128)) * JR_LOG_SWEEPS);
+  j.lay.j32_off = al((n * jacobi_ld<float>(mmax) + 1) / 2);
+  j.lay.vb64_off = al(n * ld + n + CL_MAX * 4);
+  j.lay.q_off[0] = al(mps_size(3, mmax));                  // the vectors, as the job's dst
+  j.lay.q_off[1] = al(4);                                  // its bonds (ints)
+  return j.lay.total = off;
+}
+
+// scratch: plan_gram_eig's bytes in doubles; h_job (on the host) stays until d_job is written.
+void place_gram_eig(RoundJob& j, double* scratch) {
+  j.scratch = scratch;
+  j.dst.base = scratch + j.lay.q_off[0];
+  j.dst.ranks = (int*)(scratch + j.lay.q_off[1]);
+}
+
+void launch_gram_eig(const RoundJob* d_job, const double* G, int m, double* U, int chi, double delta2, int ncols_cap,
+                     int* r_out, int* status, cudaStream_t st) {
+  cudaFuncSetAttribute(gram_eig_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)round_smem_bytes());
+  cudaFuncSetAttribute(gram_eig_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+  cudaLaunchConfig_t cfg = {};
+  cfg.blockDim = dim3(RT, 1, 1);
+  cfg.dynamicSmemBytes = round_smem_bytes();
+  cfg.stream = st;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.y = 1;
+  at[0].val.clusterDim.z = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  // the widest cluster that this device can hold (below ~32 columns the exchanges
+  // among 16 CTAs would cost more than the work)
+  int P = m < 8 ? 1 : m < 32 ? 4 : CL_MAX;
+  for (; P > 1; P /= 2) {
+    at[0].val.clusterDim.x = P;
+    cfg.gridDim = dim3(P, 1, 1);
+    int n = 0;
+    if (cudaOccupancyMaxActiveClusters(&n, gram_eig_kernel, &cfg) == cudaSuccess && n > 0) break;
+    cudaGetLastError();
+  }
+  at[0].val.clusterDim.x = P;
+  cfg.gridDim = dim3(P, 1, 1);
+  cudaLaunchKernelEx(&cfg, gram_eig_kernel, d_job, G, m, U, chi, delta2, ncols_cap, r_out, status);
+}
+
 template <typename T>
 __global__ void __launch_bounds__(RT) round_kernel(const RoundJob* __restrict__ jobs, int L_arg,
                                                    int n_bits_arg, const T* __restrict__ masks_arg,

@@ -1,6 +1,7 @@
-"""Dense contraction of MPS at the edges of its kernels' tiles: bonds around the
-16/32-wide steps of the digit products and the 128 up to which they are taken,
-lattices on both sides of the 64^3 from which they are, rows that are not finite."""
+"""Dense contraction of MPS and TT-SVD of dense fields at the edges of their kernels'
+tiles: bonds around the 16/32-wide steps of the digit products and the 128 up to
+which they are taken, lattices on both sides of the 64^3 from which they are, rows
+that are not finite; eigenproblems below, at and beyond 128 columns."""
 import numpy as np
 import pytest
 
@@ -94,3 +95,30 @@ def test_output_fields_sum_the_populations(tl):
         j = np.tensordot(c[:, d].astype(float), f, 1) + (0.5e-5 if d == 0 else 0.0)
         assert np.abs(u[d] - j / r).max() <= 1e-13
     sim.close()
+
+
+@pytest.mark.parametrize("n,bond,chi,prec", [(2, 2, 2, 0), (4, 3, 3, 0), (4, 20, 16, 0), (5, 48, 48, 0), (5, 64, 64, 1),
+                                             (6, 90, 80, 0)])
+def test_from_dense_bound(tl, n, bond, chi, prec):
+    """TT-SVD with a rank cap: cores of orthonormal columns, and an error of at most the
+    root of the summed squared tails of the field's unfoldings."""
+    import torch
+    L = 3 * n
+    cores = synth.random_mps(L, synth.feasible_ranks(L, bond), 7 + bond)
+    x = field(cores)
+    x /= np.linalg.norm(x)
+    X = tl.from_dense(torch.tensor(x, dtype=torch.float64 if prec == 0 else torch.float32, device="cuda"), chi, chi, 0.0)
+    out = X.cores()
+    for c in out[:-1]:
+        m = np.asarray(c, dtype=np.float64).reshape(-1, c.shape[2])
+        assert np.abs(m.T @ m - np.eye(m.shape[1])).max() <= (1e-12 if prec == 0 else 1e-5)
+    err = np.linalg.norm(field([np.asarray(c, dtype=np.float64) for c in out]) - x)
+    t = q.encode(x).reshape(-1)
+    tails = 0.0
+    for k in range(1, L):
+        m = t.reshape(2 ** k, -1)
+        s2 = np.linalg.eigvalsh(m @ m.T if m.shape[0] <= m.shape[1] else m.T @ m)[::-1]
+        tails += max(0.0, s2[chi:].sum())
+    # what the Gram matrices cannot resolve: 64 eps m per bond, squared norms
+    floor = (L - 1) * 64 * 2.3e-16 * 2 * chi
+    assert err ** 2 <= tails * (1 + 1e-6) + floor + (1e-9 if prec else 0.0)
