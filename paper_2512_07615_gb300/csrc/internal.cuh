@@ -106,8 +106,9 @@ struct RoundLayout {
   size_t w_off, m_off, r_off, c_off, jw_off, jv_off, us_off, rz_off, qw_off, total;
   size_t jw64_off, jv64_off;  // FP64 Jacobi matrices (in elements of T; = jw/jv for T = double)
   // refined FP64 SVDs (RoundJob::refine): rotations of the FP32 sweeps, their
-  // product (floats), a second V with the column norms and the CTAs' maxima
-  size_t log_off, j32_off, vb64_off;
+  // product (floats), a second V with the column norms and the CTAs' maxima, and W
+  // and V of FP32 sweeps over the cluster
+  size_t log_off, j32_off, vb64_off, wide_off;
 };
 
 // Learned-rank rounding state shared by all jobs of a launch (nullable parts).

@@ -275,7 +275,7 @@ __device__ void householder_qr_par(T* A, int m, int n, int lda, T* Q, int ldq, T
 // on columns stored contiguously, with a half-warp per column pair so that a
 // 1024-thread CTA keeps 64 pairs in flight.  Columns have stride ldw >= len.
 template <typename T>
-__device__ int jacobi_cols_hw(T* Wm, int ldw, T* V, int ldv, int ncol, int len, int maxsw) {
+__device__ __noinline__ int jacobi_cols_hw(T* Wm, int ldw, T* V, int ldv, int ncol, int len, int maxsw) {
   for (int idx = threadIdx.x; idx < ncol * ncol; idx += blockDim.x)
     V[(size_t)(idx / ncol) * ldv + idx % ncol] = (idx / ncol == idx % ncol) ? (T)1 : (T)0;
   __shared__ int s_rot;

@@ -44,7 +44,7 @@
 
 namespace tn {
 
-static constexpr int RF_KC = 32;         // rows of k that at least are staged at a time
+static constexpr int RF_KC = 8;          // rows of k that at least are staged at a time
 static constexpr int RF_STEPS = 12;      // steps V <- V (I + E) at most
 static constexpr int RF_PASSES = 2;      // FP32 Jacobis of W at most
 static constexpr int RF_MIN = 6;         // columns from which it is taken: below, the few rounds of the sweeps cost less
@@ -210,12 +210,14 @@ struct RefineMem {
   float* stat;             // [2][CL_MAX][4] maxima of every CTA
   float2* log;
   int ldv, ldw, ldj;
+  int turn;                // meetings so far (the slots of stat alternate)
 };
 
 // All CTAs meet; the maxima over the cluster of the four values v (thread-uniform
-// per CTA) come back in v.  `turn` alternates the slots.
+// per CTA) come back in v.
 template <typename N>
-__device__ __forceinline__ bool rf_meet_max(ClusterCtx& cc, const RefineMem<N>& m, float (&v)[4], int& turn) {
+__device__ __forceinline__ bool rf_meet_max(ClusterCtx& cc, RefineMem<N>& m, float (&v)[4]) {
+  int& turn = m.turn;
   if (threadIdx.x == 0) __stcg((float4*)(m.stat + ((size_t)(turn & 1) * CL_MAX + cc.rank) * 4), make_float4(v[0], v[1], v[2], v[3]));
   if (!cl_sync(cc)) return false;
   const int c = threadIdx.x & 15;
@@ -263,7 +265,6 @@ __device__ __noinline__ int rf_refine(ClusterCtx& cc, RefineMem<N>& m, int n, in
   const size_t fixed = rf_fixed(n, len, cc.P);
   N* st = (N*)(wa + fixed);
   const size_t rm = (size_t)room - fixed;
-  int turn = 0;
   bool last = false;
   int passes = 0;
   auto own = [&](const N* M, int ld, int rows) {           // blk <- the own columns of M
@@ -350,7 +351,7 @@ __device__ __noinline__ int rf_refine(ClusterCtx& cc, RefineMem<N>& m, int n, in
     }
     mt = (tied ? 1.f : 0.f) + (large ? 2.f : 0.f);
     float s[4] = {rf_block_max(mr, s_red), rf_block_max(mt, s_red), rf_block_max(mx, s_red), rf_block_max(dev, s_red)};
-    if (!rf_meet_max(cc, m, s, turn)) return RF_DEAD;
+    if (!rf_meet_max(cc, m, s)) return RF_DEAD;
     bool only_r = !go_on;                                  // E = R / 2 only
     if (!only_r && s[1] >= 2.f) {
       if (passes >= RF_PASSES) {
@@ -396,6 +397,62 @@ __device__ __noinline__ int rf_refine(ClusterCtx& cc, RefineMem<N>& m, int n, in
     if (only_r) go_on = false;                             // until V is orthonormal
     else last = fine;
   }
+}
+
+// W = X V carries the rounding of the whole X in its small columns, so their cosines are
+// not below ~1e-16 s_0 / s_j (FP64) whatever V is, while Jacobi rotations of W would keep them
+// small.  Where the directions of W are the orthonormal result (X is C^T), the columns are
+// made orthogonal: from every column go its parts along the larger ones (first order, at most
+// four times; the larger ones are left as they are), which changes W by those cosines
+// times s_j, its own rounding.  low: squared norms (relative to the largest) of columns
+// that are all rounding; they are left out.  False: this CTA has given up.
+template <typename N>
+__device__ __noinline__ bool rf_polish(ClusterCtx& cc, RefineMem<N>& m, int n, int len, float low, float tol2, int at,
+                                       int room) {
+  extern __shared__ __align__(16) unsigned char smem[];
+  unsigned char* wa = smem + at;
+  __shared__ float s_red[32];
+  const int v0 = cc.rank * n / cc.P, vi = (cc.rank + 1) * n / cc.P - v0;
+  const int big = imax(n, len), vmax = (n + cc.P - 1) / cc.P;
+  N* blk = (N*)wa;
+  N* nr = blk + (size_t)big * vmax;
+  float* F = (float*)(nr + n);
+  const size_t fixed = rf_fixed(n, len, cc.P);
+  N* st = (N*)(wa + fixed);
+  const size_t rm = (size_t)room - fixed;
+  for (int i = threadIdx.x; i < n; i += blockDim.x) nr[i] = __ldcg(m.nrm + i);
+  for (int j = threadIdx.x >> 5; j < vi; j += blockDim.x >> 5)
+    for (int k = threadIdx.x & 31; k < len; k += 32) blk[(size_t)j * len + k] = __ldcg(m.W + (size_t)(v0 + j) * m.ldw + k);
+  __syncthreads();
+  float nmax = 0.f;
+  for (int i = threadIdx.x & 31; i < n; i += 32) nmax = fmaxf(nmax, rf_f(nr[i]));
+  for (int o = 16; o > 0; o >>= 1) nmax = fmaxf(nmax, __shfl_xor_sync(0xffffffffu, nmax, o));
+  const float least = low * nmax;
+  for (int it = 0; it < 4; ++it) {
+    float mx = 0.f;
+    rf_gemm<N>(n, vi, len, [&](int k, int i) { return __ldcg(m.W + (size_t)i * m.ldw + k); }, true, blk, len, st, rm,
+               [&](int i, int j, N s) {
+                 const int c = v0 + j;
+                 const float si = rf_f(nr[i]), sc = rf_f(nr[c]), g = rf_f(s);
+                 float f = 0.f;
+                 if (i != c && si > least && sc > least) {
+                   const float cs = g * rsqrtf(si) * rsqrtf(sc), c2 = cs * cs;
+                   mx = fmaxf(mx, c2);
+                   if (c2 > 0.25f * tol2 && (si > sc || (si == sc && i < c))) f = -g / si;
+                 }
+                 F[(size_t)j * n + i] = f;
+               });
+    float s[4] = {rf_block_max(mx, s_red), 0.f, 0.f, 0.f};
+    if (!rf_meet_max(cc, m, s)) return false;
+    if (s[0] <= tol2) break;
+    rf_gemm<float>(len, vi, n, [&](int k, int i) { return rf_f(__ldcg(m.W + (size_t)k * m.ldw + i)); }, false, F, n, (float*)st, rm,
+                   [&](int i, int j, float v) { blk[(size_t)j * len + i] = rf_add(blk[(size_t)j * len + i], v); });
+    if (!cl_sync(cc)) return false;                        // W has been read everywhere
+    for (int j = threadIdx.x >> 5; j < vi; j += blockDim.x >> 5)
+      for (int k = threadIdx.x & 31; k < len; k += 32) __stcg(m.W + (size_t)(v0 + j) * m.ldw + k, blk[(size_t)j * len + k]);
+    if (!cl_sync(cc)) return false;
+  }
+  return true;
 }
 
 }  // namespace tn

@@ -13,6 +13,7 @@
 
 #include "cluster.cuh"
 #include "jacobi_reg.cuh"
+#include "jacobi_wide.cuh"
 #include "linalg.cuh"
 #include "qr_reg.cuh"
 #include "refine64.cuh"
@@ -108,6 +109,13 @@ void plan_round_job(RoundJob& j, int L, int n_bits, size_t eb) {
     j.lay.log_off = al(2 * lg * JR_LOG_SWEEPS / fpe);
     j.lay.j32_off = al((j32 + fpe - 1) / fpe);
     j.lay.vb64_off = al((2 * vb + CL_MAX * 8) / fpe);
+    size_t wide = 0;                               // floats
+    for (int k = 0; k < L; ++k) {
+      const int rn = imin(j.chi, j.qb[k + 1]);
+      const int ncol = imin(j.qb[k], 2 * rn), len = imax(j.qb[k], 2 * rn);
+      if (!jacobi_reg_fits(ncol, len)) wide = std::max(wide, jacobi_wide_floats(ncol, len));
+    }
+    j.lay.wide_off = al((wide + fpe - 1) / fpe);
   }
   j.lay.total = off;
 }
@@ -317,13 +325,6 @@ __device__ __forceinline__ S sum4(const S* x, int n, int s) {
   return (a0 + a1) + (a2 + a3);
 }
 
-// round-robin pair p of round rnd over np (even) indices, a < b
-__device__ __forceinline__ void rr_pair(int rnd, int p, int np, int& a, int& b) {
-  if (p == 0) { a = rnd; b = np - 1; }
-  else { a = (rnd + p) % (np - 1); b = (rnd - p + (np - 1)) % (np - 1); }
-  if (a > b) { const int t = a; a = b; b = t; }
-}
-
 // Column norms of the S-typed rows Wl over the cluster, in S arithmetic:
 // every CTA sums its rows, sends the partial sums to every CTA, and every CTA
 // adds them in rank order (the same values in every CTA).  Ends with nrm[]
@@ -488,10 +489,14 @@ __device__ __forceinline__ bool rows_angle(double al, double be, double g, doubl
 // every CTA stops at the same sweep.  Returns the sweeps used; *converged
 // tells whether the rule was met within maxsw sweeps.
 template <typename S>
-__device__ int rows_sweeps(ClusterCtx& cc, const RowsLayout& R, unsigned char* wa, S* Wl, double* Vl, int ncol,
+__device__ __noinline__ int rows_sweeps(ClusterCtx& cc_, const RowsLayout& R_, unsigned char* wa, S* Wl, double* Vl, int ncol,
                            int li, int vi, int maxsw, S tol2, unsigned* nrot, double* phase_acc, bool* converged,
                            int* rounds_out = nullptr) {
   static_assert(sizeof(S) == 8, "the cluster sweeps run on FP64 rows");
+  // in registers: behind the references they are in local memory, read again in each of
+  // the exchanges that a round is made of
+  ClusterCtx cc = cc_;
+  const RowsLayout R = R_;
   __shared__ float s_mrel[32];
   RxClock rx(phase_acc);
   unsigned q = 0;                                  // rounds so far (exchange buffer parity)
@@ -594,6 +599,7 @@ __device__ int rows_sweeps(ClusterCtx& cc, const RowsLayout& R, unsigned char* w
   }
   if (phase_acc && threadIdx.x == 0) phase_acc[PH_ROUNDS64] += rounds;
   if (rounds_out) *rounds_out = rounds;
+  cc_ = cc;
   if (cc.dead) { *converged = false; return maxsw; }
   return sweep;
 }
@@ -704,6 +710,7 @@ __device__ inline void rows_xv(const RowsLayout& R, unsigned char* wa, const T* 
   __syncthreads();
 }
 
+static constexpr int SW_WIDE = -3;
 // FP64 one-sided Jacobi SVD of the centre matrix C (m x n, T, global) with the
 // rows of the Jacobi matrices split over the CTAs of the cluster and held in
 // shared memory.  X = the columns of C (n <= m) or of C^T, scaled by scl;
@@ -716,7 +723,9 @@ __device__ inline void rows_xv(const RowsLayout& R, unsigned char* wa, const T* 
 //   CTA forms its rows of their product V0 from the log, and rf_refine takes V0 to an
 //   orthonormal V with W = X V and orthogonal columns, to 48 (FP32 data) or 53 bits;
 //   the FP64 sweeps run only where it could not finish, from the V it reached;
-// -1 (FP32 data beyond the register Jacobi): the leader's V0 is in the job's scratch;
+// SW_WIDE: the same with FP32 sweeps over the cluster, V along (jacobi_wide), where X
+//   does not fit one CTA's registers;
+// -1 (FP32 data beyond that too): the leader's V0 is in the job's scratch;
 //   one FP64 Newton-Schulz step, spread over the CTAs by blocks of columns, makes it
 //   orthogonal to ~1e-12, W = X V is formed in FP64 and the FP64 sweeps finish;
 // -2, and FP64 data: FP64 sweeps from W = X, V = I.
@@ -728,7 +737,7 @@ __device__ inline void rows_xv(const RowsLayout& R, unsigned char* wa, const T* 
 // returns the kept rank (0 if it exceeds the bond capacity), the FP64
 // sweeps, whether their limit was reached, and the FP64 FLOPs executed.
 template <typename T>
-__device__ int svd64_rows(ClusterCtx& cc, const RoundJob& J, int L, int k, int m, int n, double scl, double delta,
+__device__ __noinline__ int svd64_rows(ClusterCtx& cc, const RoundJob& J, int L, int k, int m, int n, double scl, double delta,
                           int maxsw, int sw32, int* sweeps_out, bool* noconv, double* exec_flops = nullptr,
                           double* phase_acc = nullptr) {
   constexpr bool two_phase = sizeof(T) == 4;
@@ -756,8 +765,25 @@ __device__ int svd64_rows(ClusterCtx& cc, const RoundJob& J, int L, int k, int m
   auto xat = [&](int i, int kk) -> double { return scl * (double)__ldcg(trans ? C + (size_t)i * n + kk : C + (size_t)kk * n + i); };
   const int ld1 = jacobi_ld<double>(ncol);
   int state = RF_SWEEPS;
-  if (sw32 >= 0) {
-    // start from the leader's logged FP32 sweeps, refine by products
+  // squared norms relative to the largest below which a refined W is rounding only
+  constexpr float low = two_phase ? 1e-22f : 1e-27f;
+  if (sw32 >= 0 || sw32 == SW_WIDE) {
+    // start from FP32 sweeps, refine by products
+    const bool wide = sw32 == SW_WIDE;
+    const int ldw32 = wide ? jacobi_wide_ldw(len) : jacobi_reg_ld(len);
+    float* Wg = (float*)(scr + J.lay.wide_off);
+    float* Vg = Wg + (size_t)jacobi_wide_cols(ncol) * ldw32;
+    // FP32 sweeps of x(i, j) over the cluster, Vg their product
+    auto sweep_wide = [&](auto&& x) -> int {
+      const int nc = 2 * jacobi_wide_ctas(cc.P) * jacobi_wide_block(ncol, cc.P);
+      for (int j = cc.rank; j < nc; j += cc.P) {
+        for (int i = threadIdx.x; i < ldw32; i += blockDim.x)
+          __stcg(Wg + (size_t)j * ldw32 + i, j < ncol && i < len ? x(i, j) : 0.f);
+        for (int i = threadIdx.x; i < JW_COLS; i += blockDim.x) __stcg(Vg + (size_t)j * JW_COLS + i, i == j && j < ncol ? 1.f : 0.f);
+      }
+      if (!cl_sync(cc)) return maxsw;
+      return jacobi_wide(cc, Wg, Vg, ncol, len, imin(maxsw, JW_SWEEPS), (float*)wa);
+    };
     const long long t0 = clock64();
     using N = typename std::conditional<two_phase, float2, double>::type;
     RefineMem<N> rm;
@@ -771,14 +797,27 @@ __device__ int svd64_rows(ClusterCtx& cc, const RoundJob& J, int L, int k, int m
     rm.ldj = jacobi_ld<float>(ncol);
     rm.nrm = rm.V2 + (size_t)ncol * ld1;
     rm.log = (float2*)(scr + J.lay.log_off);
-    jacobi_reg_apply(rm.log, sw32, ncol, v0, vi, rm.V, ld1, (float2*)wa);
+    rm.turn = 0;
+    if (wide) {
+      sw32 = sweep_wide([&](int i, int j) { return (float)xat(i, j); });
+      for (int idx = threadIdx.x; idx < ncol * vi; idx += blockDim.x)
+        __stcg(rm.V + (size_t)(v0 + idx / ncol) * ld1 + idx % ncol, rf_make<N>(__ldcg(Vg + (size_t)(v0 + idx / ncol) * JW_COLS + idx % ncol)));
+    } else {
+      jacobi_reg_apply(rm.log, sw32, ncol, v0, vi, rm.V, ld1, (float2*)wa);
+    }
     cl_sync(cc);
     // one more FP32 Jacobi, of W: the leader's sweeps, their product over the cluster
     auto jacobi = [&]() -> bool {
       int sw = 0;
+      if (wide) {
+        sweep_wide([&](int i, int j) { return 1048576.f * rf_f(__ldcg(rm.W + (size_t)j * rm.ldw + i)); });
+        for (int idx = threadIdx.x; idx < ncol * vi; idx += blockDim.x)
+          __stcg(rm.J + (size_t)(v0 + idx / ncol) * rm.ldj + idx % ncol, __ldcg(Vg + (size_t)(v0 + idx / ncol) * JW_COLS + idx % ncol));
+        return cl_sync(cc);
+      }
       if (cc.rank == 0) {
         float* Wf = (float*)wa;
-        const int ldw32 = jacobi_reg_ld(len), ncp = jacobi_reg_cols(ncol);
+        const int ncp = jacobi_reg_cols(ncol);
         for (int idx = threadIdx.x; idx < ncp * ldw32; idx += blockDim.x) {
           const int jj = idx / ldw32, i = idx % ldw32;
           // 2^20: columns down to 1e-18 of the scale are above the Jacobi's floor
@@ -800,7 +839,8 @@ __device__ int svd64_rows(ClusterCtx& cc, const RoundJob& J, int L, int k, int m
     const float tol2r = (two_phase ? 256.f : 1.f) * (float)(tol64 * tol64);
     state = rf_refine<N>(cc, rm, ncol, len, sw32 < maxsw, xn, trans, trans, tol2r,
                          two_phase ? 2e-13f : 2e-15f, two_phase ? 2e-6f : 2e-9f, two_phase ? 1e-11f : 1e-14f,
-                         two_phase ? 1e-22f : 1e-27f, SM_SMALL, SM_WORK, jacobi);
+                         two_phase ? 1e-22f : 1e-30f, SM_SMALL, SM_WORK, jacobi);
+    if (state == RF_DONE && !trans && !rf_polish<N>(cc, rm, ncol, len, low, tol2r, SM_SMALL, SM_WORK)) state = RF_DEAD;
     if (phase_acc && threadIdx.x == 0) phase_acc[PH_NS] += (double)(clock64() - t0);
     const long long t1 = clock64();
     for (int idx = threadIdx.x; idx < ncol * vi; idx += blockDim.x) {
@@ -864,37 +904,48 @@ __device__ int svd64_rows(ClusterCtx& cc, const RoundJob& J, int L, int k, int m
   }
   // exact norms -> singular values, order and rank (identical in every CTA);
   // non-finite values order last and are reported
-  rows_norms<double>(cc, R, wa, W, ncol, li);
-  for (int j = threadIdx.x; j < ncol; j += blockDim.x) {
-    const double sv = sqrt(nrm[j]) / scl;
-    if (!(sv >= 0.0) || isinf(sv)) { sig[j] = -1.0; atomicOr(cc.status, ST_NAN); }
-    else sig[j] = sv;
-  }
-  __syncthreads();
-  for (int j = threadIdx.x; j < ncol; j += blockDim.x) {
-    int rank = 0;
-    const double sj = sig[j];
-    for (int o = 0; o < ncol; ++o) rank += (sig[o] > sj) || (sig[o] == sj && o < j);
-    perm[rank] = j;
-  }
-  __syncthreads();
   __shared__ int s_r;
-  if (threadIdx.x == 0) {
-    const int rmax = imin(J.chi, ncol);
-    double tail2 = 0.0;
-    for (int p = ncol - 1; p >= 1; --p) {
-      const double sv = sig[perm[p]];
-      tail2 += sv * sv;
-      tail[2 + p] = tail2;
+  for (bool again = false;; again = true) {
+    rows_norms<double>(cc, R, wa, W, ncol, li);
+    for (int j = threadIdx.x; j < ncol; j += blockDim.x) {
+      const double sv = sqrt(nrm[j]) / scl;
+      if (!(sv >= 0.0) || isinf(sv)) { sig[j] = -1.0; atomicOr(cc.status, ST_NAN); }
+      else sig[j] = sv;
     }
-    int rr = rmax;
-    for (int qq = 1; qq <= rmax; ++qq) {
-      const double t2 = (qq < ncol) ? tail[2 + qq] : 0.0;
-      if (sqrt(t2) <= delta) { rr = qq; break; }
+    __syncthreads();
+    for (int j = threadIdx.x; j < ncol; j += blockDim.x) {
+      int rank = 0;
+      const double sj = sig[j];
+      for (int o = 0; o < ncol; ++o) rank += (sig[o] > sj) || (sig[o] == sj && o < j);
+      perm[rank] = j;
     }
-    s_r = rr > bond_cap(L, J.dst.cap, k) ? 0 : rr;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      const int rmax = imin(J.chi, ncol);
+      double tail2 = 0.0;
+      for (int p = ncol - 1; p >= 1; --p) {
+        const double sv = sig[perm[p]];
+        tail2 += sv * sv;
+        tail[2 + p] = tail2;
+      }
+      int rr = rmax;
+      for (int qq = 1; qq <= rmax; ++qq) {
+        const double t2 = (qq < ncol) ? tail[2 + qq] : 0.0;
+        if (sqrt(t2) <= delta) { rr = qq; break; }
+      }
+      s_r = rr > bond_cap(L, J.dst.cap, k) ? 0 : rr;
+    }
+    __syncthreads();
+    // kept columns of W that are all rounding have no directions (a tolerance below the
+    // refinement's resolution): the sweeps orthogonalise them like any others
+    if (again || state != RF_DONE || trans || s_r < 1 || cc.dead) break;
+    const double s0 = sig[perm[0]], sl = sig[perm[s_r - 1]];
+    if (sl * sl > (double)low * s0 * s0) break;
+    __syncthreads();
+    sw = rows_sweeps<double>(cc, R, wa, W, Vl, ncol, li, vi, maxsw, tol64 * tol64, &s_nrot, phase_acc, &conv, &rounds);
+    *sweeps_out = sw;
+    *noconv = !conv || cc.dead;
   }
-  __syncthreads();
   const int r = s_r;
   if (r > 0 && !cc.dead) {
     if (trans) {
@@ -978,13 +1029,15 @@ __device__ __noinline__ int svd64_site(const RoundJob& J, int L, int k, const T*
     int sw32 = 0;
     bool logged = false;
     const bool plain = ncol < RF_MIN;             // FP64 sweeps from V = I
-    if (!plain && (sizeof(T) == 4 || J.refine)) {
+    const bool refine = J.refine && rf_bytes(ncol, len, cc.P) <= (size_t)SM_WORK;
+    const bool wide = refine && !jacobi_reg_fits(ncol, len) && jacobi_wide_fits(ncol, len, cc.P);
+    if (!plain && !wide && (sizeof(T) == 4 || J.refine)) {
       // FP32 sweeps on X by this CTA alone (its own stopping rule, a
       // sweep limit, convergence not required).  In registers where X fits: W only,
       // the rotations logged for the cluster to form V0 (a row of V0 per half-warp,
       // ~1/16 of the sweeps' time on 16 CTAs, where carrying V along would double
       // the sweeps' work)
-      if (J.refine && jacobi_reg_fits(ncol, len) && rf_bytes(ncol, len, cc.P) <= (size_t)SM_WORK) {
+      if (refine && jacobi_reg_fits(ncol, len)) {
         float* Wf = (float*)work;
         const int ldw32 = jacobi_reg_ld(len), ncp = jacobi_reg_cols(ncol);
         for (int idx = threadIdx.x; idx < ncp * ldw32; idx += blockDim.x) {
@@ -1019,12 +1072,12 @@ __device__ __noinline__ int svd64_site(const RoundJob& J, int L, int k, const T*
       if (threadIdx.x == 0) pc.acc[PH_SWEEPS32] += sw32;
       pc.lap(PH_J32);
     }
-    cl_command(cc, 2, ncol, len, maxsw, m, n, k, delta, scl, logged ? sw32 : plain ? -2 : -1);
+    const int start = wide ? SW_WIDE : logged ? sw32 : plain ? -2 : -1;
+    cl_command(cc, 2, ncol, len, maxsw, m, n, k, delta, scl, start);
     int sw = 0;
     bool noconv = false;
     double xfl = 0.0;
-    const int r = svd64_rows<T>(cc, J, L, k, m, n, scl, delta, maxsw, logged ? sw32 : plain ? -2 : -1, &sw, &noconv, &xfl,
-                                pc.on ? pc.acc : nullptr);
+    const int r = svd64_rows<T>(cc, J, L, k, m, n, scl, delta, maxsw, start, &sw, &noconv, &xfl, pc.on ? pc.acc : nullptr);
     pc.lap(PH_JACOBI);
     if (threadIdx.x == 0) { pc.acc[PH_SVD64_FLOPS] += svd_flops(m, n); pc.acc[PH_SVD64_EXEC] += xfl; }
     const RowsLayout R = rows_layout(ncol, len, cc.P, sizeof(T) == 4);
@@ -1972,6 +2025,7 @@ size_t plan_gram_eig(RoundJob& j, int mmax) {
   j.lay.log_off = al(jacobi_reg_log_sweep(imin(mmax, 128)) * JR_LOG_SWEEPS);
   j.lay.j32_off = al((n * jacobi_ld<float>(mmax) + 1) / 2);
   j.lay.vb64_off = al(n * ld + n + CL_MAX * 4);
+  j.lay.wide_off = jacobi_reg_fits(mmax, mmax) ? 0 : al((jacobi_wide_floats(mmax, mmax) + 1) / 2);
   j.lay.q_off[0] = al(mps_size(3, mmax));                  // the vectors, as the job's dst
   j.lay.q_off[1] = al(4);                                  // its bonds (ints)
   return j.lay.total = off;
