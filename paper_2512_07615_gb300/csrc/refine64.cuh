@@ -354,10 +354,9 @@ __device__ __noinline__ int rf_refine(ClusterCtx& cc, RefineMem<N>& m, int n, in
     if (!rf_meet_max(cc, m, s)) return RF_DEAD;
     bool only_r = !go_on;                                  // E = R / 2 only
     if (!only_r && s[1] >= 2.f) {
-      if (passes >= RF_PASSES) {
-        only_r = true;
+      if (passes >= RF_PASSES || step >= RF_STEPS) {
+        only_r = true;                                     // V is handed on orthonormal
       } else if (s[3] > ready) {
-        if (step >= RF_STEPS) return RF_SWEEPS;
         for (int idx = threadIdx.x; idx < n * vi; idx += blockDim.x) E[idx] = 0.5f * R[idx];
         correct();
         if (!cl_sync(cc)) return RF_DEAD;
@@ -393,7 +392,8 @@ __device__ __noinline__ int rf_refine(ClusterCtx& cc, RefineMem<N>& m, int n, in
     swap();
     // small enough: what is left after this step is of order E^2, W = X V once more
     const bool fine = (only_r ? s[3] : s[2]) <= small;
-    if (only_r && (fine || step >= RF_STEPS + 3)) return RF_SWEEPS;
+    // (|R| squares from step to step, from 0.1 at most: 1e-2, 1e-4, 1e-8, 1e-16)
+    if (only_r && (fine || step >= RF_STEPS + 8)) return RF_SWEEPS;
     if (only_r) go_on = false;                             // until V is orthonormal
     else last = fine;
   }
