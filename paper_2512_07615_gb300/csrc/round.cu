@@ -435,8 +435,44 @@ __device__ __forceinline__ void renorm64(float cf, float sf, double& c, double& 
 // s = t c; else the FP32 (c, s) renormalised in FP64 (renorm64).  The new
 // norms are al - t g and be + t g (exact for the exact root; recomputed every
 // sweep); rel2 = g^2 / (al be) for the stopping rule.
+// A warp's FP64 instruction takes 64 cycles of its scheduler (0.5 lanes a clock), and a
+// round waits for this chain: 30 of them took 4 k of a round's 9 k cycles.  So where al, be
+// and g are within 2^+-100 and al, be within 2^100 of each other, the test and the quotient
+// are FP32, conversions of normal numbers move bits, and ten FP64 instructions are left:
+// 4.0 k -> 3.2 k cycles.
+__device__ __forceinline__ float narrow_bits(double x) {    // |x| in 2^+-126, truncated
+  const unsigned h = (unsigned)__double2hiint(x), l = (unsigned)__double2loint(x);
+  return __uint_as_float((h & 0x80000000u) | (((h & 0x7fffffffu) - 0x38000000u) << 3) | (l >> 29));
+}
+__device__ __forceinline__ double widen_bits(float x) {     // a normal number
+  const unsigned u = __float_as_uint(x);
+  return __hiloint2double((int)((u & 0x80000000u) | (((u & 0x7fffffffu) >> 3) + 0x38000000u)), (int)(u << 29));
+}
 __device__ __forceinline__ bool rows_angle(double al, double be, double g, double tol2, double& cw, double& sw,
                                            double& na, double& nb, float& rel2) {
+  const int xa = __double2hiint(al) >> 20, xb = __double2hiint(be) >> 20, xg = (__double2hiint(g) >> 20) & 0x7ff;
+  if (xa > 923 && xa < 1123 && xb > 923 && xb < 1123 && xg > 923 && xg < 1123 && xa - xb < 100 && xb - xa < 100) {
+    const float gf = narrow_bits(g);
+    const float cs = fabsf(gf) * (rsqrtf(narrow_bits(al)) * rsqrtf(narrow_bits(be)));
+    if (!(cs > sqrtf((float)tol2))) return false;
+    rel2 = cs * cs;
+    const float z = (float)(be - al) / (2.f * gf), az = fabsf(z);
+    const float tf = copysignf(az > 1e18f ? 0.5f / az : 1.f / (az + sqrtf(fmaf(z, z, 1.f))), z);
+    const double t = widen_bits(tf);                        // at least 2^-100: normal
+    if (fabsf(tf) < 6.1035156e-05f) {
+      cw = fma(-0.5 * t, t, 1.0);                           // c^2 + s^2 = 1 - 3 t^4 / 4 + ...
+      sw = t * cw;
+    } else {
+      const float cf = rsqrtf(fmaf(tf, tf, 1.f));
+      const double c0 = widen_bits(cf), s0 = widen_bits(cf * tf);
+      const double dr = fma(c0, c0, fma(s0, s0, -1.0)), h = fma(dr, fma(0.375, dr, -0.5), 1.0);
+      cw = c0 * h;
+      sw = s0 * h;
+    }
+    na = fma(-t, g, al);
+    nb = fma(t, g, be);
+    return true;
+  }
   const double gg = g * g, ab = al * be;
   if (g == 0.0 || !(al > 1e-250) || !(be > 1e-250) || gg <= tol2 * ab) return false;
   rel2 = (float)gg / (float)ab;                         // +inf if al be leaves the FP32 range
@@ -541,9 +577,13 @@ __device__ __noinline__ int rows_sweeps(ClusterCtx& cc_, const RowsLayout& R_, u
         // the partials of pair p in rank order: lane l adds ranks l, l+4, ...,
         // then the four lanes combine (the same order in every CTA)
         S g = 0;
-        for (int c = l; c < cc.P; c += 4) g += xq[(size_t)p * cc.P + c];
-        g += __shfl_xor_sync(grp, g, 1, 4);
-        g += __shfl_xor_sync(grp, g, 2, 4);
+        if (cc.P == 1) {
+          g = xq[p];
+        } else {
+          for (int c = l; c < cc.P; c += 4) g += xq[(size_t)p * cc.P + c];
+          g += __shfl_xor_sync(grp, g, 1, 4);
+          g += __shfl_xor_sync(grp, g, 2, 4);
+        }
         if (l != 0) continue;
         int a, b;
         rr_pair(rnd, p, np, a, b);
@@ -711,6 +751,14 @@ __device__ inline void rows_xv(const RowsLayout& R, unsigned char* wa, const T* 
 }
 
 static constexpr int SW_WIDE = -3;
+// Centre matrices whose sweeps the leader runs alone, as a cluster of one: the exchanges of a
+// round (~3 k of its 9 k cycles) cost more than the other CTAs' FP64 units bring for a
+// few columns, and below ~16 columns the refinement of FP64 data costs more than
+// the sweeps.  Ten channel steps (16^3, FP64): 62.2 -> 56.6 ms on average (58.7 with cluster
+// sweeps throughout), with 12 columns 57.9, 24 as 16, 32 worse for the roundings.  FP32 data
+// are refined from RF_MIN columns on (16 columns alone: 128^3 sums 55 -> 61 ms).
+static constexpr int SOLO_LEN = 128;
+template <typename T> struct Solo { static constexpr int cols = sizeof(T) == 8 ? 16 : RF_MIN - 1; };
 // FP64 one-sided Jacobi SVD of the centre matrix C (m x n, T, global) with the
 // rows of the Jacobi matrices split over the CTAs of the cluster and held in
 // shared memory.  X = the columns of C (n <= m) or of C^T, scaled by scl;
@@ -1023,12 +1071,17 @@ __device__ __noinline__ int svd64_site(const RoundJob& J, int L, int k, const T*
   __syncthreads();
   const double scl = sh.tau[1];
   const int maxsw = J.max_sweeps > 0 ? J.max_sweeps : 60;
-  if (!in_smem && cc.P > 1 && rows_layout(ncol, len, cc.P, sizeof(T) == 4).total <= (size_t)SM_WORK) {
+  // few columns: the sweeps of this CTA alone (a cluster of one)
+  const bool solo = cc.P > 1 && ncol <= Solo<T>::cols && len <= SOLO_LEN;
+  ClusterCtx one = cc;
+  one.P = 1;
+  one.rank = 0;
+  if (solo || (!in_smem && cc.P > 1 && rows_layout(ncol, len, cc.P, sizeof(T) == 4).total <= (size_t)SM_WORK)) {
     // rows of the Jacobi matrices spread over the cluster, in shared memory
     pc.lap(PH_SVD_OUT);
     int sw32 = 0;
     bool logged = false;
-    const bool plain = ncol < RF_MIN;             // FP64 sweeps from V = I
+    const bool plain = solo || ncol < RF_MIN;     // FP64 sweeps from V = I
     const bool refine = J.refine && rf_bytes(ncol, len, cc.P) <= (size_t)SM_WORK;
     const bool wide = refine && !jacobi_reg_fits(ncol, len) && jacobi_wide_fits(ncol, len, cc.P);
     if (!plain && !wide && (sizeof(T) == 4 || J.refine)) {
@@ -1073,14 +1126,14 @@ __device__ __noinline__ int svd64_site(const RoundJob& J, int L, int k, const T*
       pc.lap(PH_J32);
     }
     const int start = wide ? SW_WIDE : logged ? sw32 : plain ? -2 : -1;
-    cl_command(cc, 2, ncol, len, maxsw, m, n, k, delta, scl, start);
+    if (!solo) cl_command(cc, 2, ncol, len, maxsw, m, n, k, delta, scl, start);
     int sw = 0;
     bool noconv = false;
     double xfl = 0.0;
-    const int r = svd64_rows<T>(cc, J, L, k, m, n, scl, delta, maxsw, start, &sw, &noconv, &xfl, pc.on ? pc.acc : nullptr);
+    const int r = svd64_rows<T>(solo ? one : cc, J, L, k, m, n, scl, delta, maxsw, start, &sw, &noconv, &xfl, pc.on ? pc.acc : nullptr);
     pc.lap(PH_JACOBI);
     if (threadIdx.x == 0) { pc.acc[PH_SVD64_FLOPS] += svd_flops(m, n); pc.acc[PH_SVD64_EXEC] += xfl; }
-    const RowsLayout R = rows_layout(ncol, len, cc.P, sizeof(T) == 4);
+    const RowsLayout R = rows_layout(ncol, len, solo ? 1 : cc.P, sizeof(T) == 4);
     const unsigned char* wa = (const unsigned char*)work;
     const double* sig = (const double*)(wa + R.sig);
     const int* perm = (const int*)(wa + R.perm);

@@ -1,7 +1,8 @@
-"""Roundings whose centre matrices are beyond one CTA's registers: the FP32 sweeps over
-the cluster and the refinement of their V, at the edges of the blocks (ncol just
-above 128, odd counts, up to 256; columns up to 256 and up to 512 entries) and just
-beyond them, and one within the registers, in mixed precision and FP64, against the dense FP64 sums."""
+"""FP64-accurate centre SVDs at the edges of their paths, in mixed precision and FP64,
+against the dense FP64 sums: few columns (the leader's sweeps up to 16 of them, 5 in
+mixed precision), one size within a CTA's registers, and beyond them the FP32
+sweeps over the cluster (ncol just above 128, odd counts, up to 256; columns up to 256
+and up to 512 entries) and the sizes past those."""
 import numpy as np
 import pytest
 
@@ -46,7 +47,7 @@ def flat_field(cores):
 
 
 # centre matrices at the widest bond: (sum of the operands' bonds) x 2 chi
-@pytest.mark.parametrize("bond,chi,terms", [(45, 90, 2), (65, 65, 2), (67, 67, 2), (100, 100, 2), (128, 128, 2), (70, 140, 2),
+@pytest.mark.parametrize("bond,chi,terms", [(2, 2, 2), (3, 3, 2), (8, 8, 2), (9, 9, 2), (45, 90, 2), (65, 65, 2), (67, 67, 2), (100, 100, 2), (128, 128, 2), (70, 140, 2),
                                             (90, 128, 3), (50, 200, 2), (90, 140, 3)])
 @pytest.mark.parametrize("prec", [0, 3])
 def test_rounded_sum(tl, bond, chi, terms, prec):
