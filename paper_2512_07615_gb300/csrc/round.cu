@@ -886,8 +886,8 @@ __device__ __noinline__ int svd64_rows(ClusterCtx& cc, const RoundJob& J, int L,
     // the sums of FP32 data carry 48 bits
     const float tol2r = (two_phase ? 256.f : 1.f) * (float)(tol64 * tol64);
     state = rf_refine<N>(cc, rm, ncol, len, sw32 < maxsw, xn, trans, trans, tol2r,
-                         two_phase ? 2e-13f : 2e-15f, two_phase ? 2e-6f : 2e-9f, two_phase ? 1e-11f : 1e-14f,
-                         two_phase ? 1e-22f : 1e-30f, SM_SMALL, SM_WORK, jacobi);
+                         two_phase ? 2e-13f : 1e-16f, two_phase ? 2e-6f : 2e-9f, two_phase ? 1e-11f : 1e-14f,
+                         two_phase ? 1e-22f : 1e-28f, SM_SMALL, SM_WORK, jacobi);
     if (state == RF_DONE && !trans && !rf_polish<N>(cc, rm, ncol, len, low, tol2r, SM_SMALL, SM_WORK)) state = RF_DEAD;
     if (phase_acc && threadIdx.x == 0) phase_acc[PH_NS] += (double)(clock64() - t0);
     const long long t1 = clock64();
