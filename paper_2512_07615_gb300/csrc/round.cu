@@ -989,7 +989,7 @@ __device__ __noinline__ int svd64_rows(ClusterCtx& cc, const RoundJob& J, int L,
     if (again || state != RF_DONE || trans || s_r < 1 || cc.dead) break;
     const double s0 = sig[perm[0]], sl = sig[perm[s_r - 1]];
     if (sl * sl > (double)low * s0 * s0) break;
-    __syncthreads();
+    cl_sync(cc);                                  // the norms' slots have been read everywhere
     sw = rows_sweeps<double>(cc, R, wa, W, Vl, ncol, li, vi, maxsw, tol64 * tol64, &s_nrot, phase_acc, &conv, &rounds);
     *sweeps_out = sw;
     *noconv = !conv || cc.dead;
