@@ -430,8 +430,8 @@ def cpu_threads():
 
 # ------------------------------------------------------------------ main
 def precision_desc(p):
-    svd64 = ("fp64 one-sided Jacobi (cluster of CTAs, started from fp32 sweeps made orthogonal by an fp64 "
-             "Newton-Schulz step), fp64 norms and tails")
+    svd64 = ("fp32 one-sided Jacobi refined by products over a cluster of CTAs (48-bit sums; fp64 sweeps for the "
+             "smallest and largest matrices), fp64 norms and tails")
     return {0: dict(storage="fp64", contractions="fp64 SIMT", qr="fp64", svd="fp64 one-sided Jacobi"),
             1: dict(storage="fp32", contractions="fp32 SIMT", qr="fp32 (scaled fp32 column norms)",
                     svd="fp32 one-sided Jacobi, fp64 tails"),
