@@ -1239,8 +1239,8 @@ static int macro_impl(tnlbm_sim* s, double* rho, double* u) {
   const size_t nc = (size_t)s->N * s->N * s->N;
   double *d = nullptr, *dm = nullptr, *tmp = nullptr;
   void* scr = nullptr;
-  const int capmax = std::max(s->cfg.chi_max, s->mask_node >= 0 ? s->nodes[s->mask_node].cap : 1);
-  const size_t sb = contract_scratch_bytes(s->n, capmax, sizeof(T));
+  size_t sb = contract_scratch_bytes(s->n, s->cfg.chi_max, sizeof(T));
+  if (s->mask_node >= 0) sb = std::max(sb, contract_scratch_bytes(s->n, s->nodes[s->mask_node].cap, sizeof(T)));
   auto fin = [&](int rc) { cudaFree(d); cudaFree(dm); cudaFree(tmp); cudaFree(scr); return rc; };
   if (cudaMalloc(&d, 4 * nc * sizeof(double)) != cudaSuccess || cudaMalloc(&tmp, nc * sizeof(double)) != cudaSuccess ||
       cudaMalloc(&scr, sb) != cudaSuccess) {
@@ -1249,12 +1249,15 @@ static int macro_impl(tnlbm_sim* s, double* rho, double* u) {
   }
   double *dr = d, *jx = d + nc, *jy = d + 2 * nc, *jz = d + 3 * nc;
   contract_begin(scr, s->s0);
-  for (int i = 0; i < s->lat.Q; ++i)
-    contract_moments<T>(s->nodes[s->f_state[i]], s->n, tmp, scr, sb, dr, jx, jy, jz, s->lat.c[i][0], s->lat.c[i][1],
-                        s->lat.c[i][2], i == 0, s->s0);
+  for (int i = 0; i < s->lat.Q; ++i) {
+    const int rc = contract_moments<T>(s->nodes[s->f_state[i]], s->n, tmp, scr, sb, dr, jx, jy, jz, s->lat.c[i][0],
+                                       s->lat.c[i][1], s->lat.c[i][2], i == 0, s->s0);
+    if (rc) return fin(rc);
+  }
   if (s->mask_node >= 0) {
     if (cudaMalloc(&dm, nc * sizeof(double)) != cudaSuccess) return fin(TNLBM_E_OOM);
-    contract_dense_f64<T>(s->nodes[s->mask_node], s->n, dm, scr, sb, s->s0);
+    const int rc = contract_dense_f64<T>(s->nodes[s->mask_node], s->n, dm, scr, sb, s->s0);
+    if (rc) return fin(rc);
   }
   if (u) launch_velocity(nc, dr, jx, jy, jz, dm, s->cfg.force[0], s->cfg.force[1], s->cfg.force[2], s->s0);
   if (rho) cudaMemcpyAsync(rho, dr, nc * sizeof(double), cudaMemcpyDeviceToHost, s->s0);

@@ -491,7 +491,8 @@ struct ContractPlan {
   int L, h, ld, chunks;
   size_t lm, rt, a, b, ea, eb, tops, total;      // byte offsets in the scratch, after the status word
 };
-static ContractPlan contract_plan(int n_bits, int cap) {
+// The size is no monotonic function of cap: the digits come with the caps that take them.
+static ContractPlan contract_plan(int n_bits, int cap, bool digits) {
   ContractPlan p;
   p.L = 3 * n_bits;
   p.h = p.L / 2;
@@ -502,7 +503,7 @@ static ContractPlan contract_plan(int n_bits, int cap) {
   auto take = [&](size_t bytes) { const size_t at = o; o += (bytes + 255) & ~(size_t)255; return at; };
   p.lm = take(nl * p.ld * sizeof(double));
   p.rt = take(nr * p.ld * sizeof(double));
-  if (by_digits<float>(n_bits, cap)) {
+  if (digits) {
     p.a = take(nl / JM * p.chunks * J_A * sizeof(uint16_t));
     p.b = take(nr / JN * p.chunks * J_B * sizeof(uint16_t));
     p.ea = take(nl * sizeof(int));
@@ -516,8 +517,12 @@ static ContractPlan contract_plan(int n_bits, int cap) {
 }
 
 size_t contract_scratch_bytes(int n_bits, int cap, size_t elem) {
-  (void)elem;
-  return contract_plan(n_bits, cap).total;
+  return contract_plan(n_bits, cap, elem == 4 && by_digits<float>(n_bits, cap)).total;
+}
+
+static int contract_short() {
+  set_error("the scratch of a contraction is too small");
+  return TNLBM_E_ARG;
 }
 
 // Prefix and suffix rows of X (and their digits).
@@ -551,11 +556,12 @@ static void join_digits(const MpsRef& X, int n_bits, const ContractPlan& p, unsi
 
 template <typename T, typename OutT>
 static int contract_to(const MpsRef& X, int n_bits, OutT* d_dense, void* d_scratch, size_t scratch_bytes, cudaStream_t st) {
-  const ContractPlan p = contract_plan(n_bits, X.cap);
-  if (p.total > scratch_bytes) return TNLBM_E_ARG;
+  const bool digits = by_digits<T>(n_bits, X.cap);
+  const ContractPlan p = contract_plan(n_bits, X.cap, digits);
+  if (p.total > scratch_bytes) return contract_short();
   unsigned char* scr = (unsigned char*)d_scratch;
   contract_rows<T>(X, n_bits, p, scr, st);
-  if (by_digits<T>(n_bits, X.cap) && (size_t)d_dense % 16 == 0)
+  if (digits && (size_t)d_dense % 16 == 0)
     join_digits(X, n_bits, p, scr, FieldOut<OutT>{d_dense}, st);
   else
     join_kernel<OutT><<<152 * 16, 256, 0, st>>>(X.ranks, n_bits, p.h, (const double*)(scr + p.lm), (const double*)(scr + p.rt),
@@ -594,8 +600,8 @@ template <typename T>
 int contract_moments(const MpsRef& X, int n_bits, double* tmp, void* d_scratch, size_t scratch_bytes, double* rho,
                      double* jx, double* jy, double* jz, int cx, int cy, int cz, int first, cudaStream_t st) {
   if (by_digits<T>(n_bits, X.cap)) {
-    const ContractPlan p = contract_plan(n_bits, X.cap);
-    if (p.total > scratch_bytes) return TNLBM_E_ARG;
+    const ContractPlan p = contract_plan(n_bits, X.cap, true);
+    if (p.total > scratch_bytes) return contract_short();
     contract_rows<T>(X, n_bits, p, (unsigned char*)d_scratch, st);
     join_digits(X, n_bits, p, (unsigned char*)d_scratch, MomentOut{{rho, jx, jy, jz}, {cx, cy, cz}, first}, st);
     return 0;

@@ -117,6 +117,8 @@ int contract_end(const void* d_scratch, cudaStream_t st, const char* what);
 template <typename T>
 int contract_dense(const MpsRef& X, int n_bits, T* d_dense, void* d_scratch, size_t scratch_bytes,
                    cudaStream_t st);
+// bytes that the contraction of an MPS of this cap and element size takes (not
+// monotonic in the cap: a scratch shared by several takes the largest of theirs)
 size_t contract_scratch_bytes(int n_bits, int cap, size_t elem);
 template <typename T>
 int contract_dense_f64(const MpsRef& X, int n_bits, double* d_dense, void* d_scratch, size_t scratch_bytes,
