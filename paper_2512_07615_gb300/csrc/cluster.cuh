@@ -33,7 +33,7 @@ struct ClusterCmd {
                           // global memory), 2 = row-partitioned FP64 SVD of site k
   int ncol, len, maxsw;
   int m, n, k;
-  int sw32;               // logged FP32 sweeps that start the SVD (-1: their V is in scratch)
+  int sw32;               // how the SVD starts: logged FP32 sweeps, or SW_* (rows_layout.cuh)
   double delta, scl;
 };
 

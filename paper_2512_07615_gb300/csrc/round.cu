@@ -17,12 +17,11 @@
 #include "linalg.cuh"
 #include "qr_reg.cuh"
 #include "refine64.cuh"
+#include "rows_layout.cuh"
 
 namespace tn {
 
 static constexpr int RT = 512;                      // threads per rounding CTA
-static constexpr int SM_SMALL = 41 * 1024;          // bookkeeping part of smem
-static constexpr int SM_WORK = 176 * 1024;          // work area in smem
 static constexpr int MAXK = 1024;                   // max columns of a QR / SVD
 
 size_t round_smem_bytes() { return SM_SMALL + SM_WORK; }
@@ -258,51 +257,6 @@ struct RxClock {
 };
 
 // ---------------------------------------------------------------- row-partitioned FP64 SVD
-// Work-area layout (bytes, same in every CTA of the cluster) of svd64_rows:
-// the CTA's rows of W and of V (FP64), the column norms, each pair's rotation
-// and flag, the exchange buffers of the pair inner products and of the
-// column norms, and the singular values, order and tails the rank rule
-// reads.  For FP32 data the block of G = V0^T V0 and the staged rows of V and
-// of X used by the Newton-Schulz step and by W = X V share the exchange
-// buffers' space (those run before the first exchange of the sweeps).
-struct RowsLayout {
-  int lw, lv, npairs, kc;
-  size_t wl, vl, nrm, pcw, psw, pf, gl, xb, nbuf, gb, st, xs, sig, perm, tail, total;
-};
-__host__ __device__ inline RowsLayout rows_layout(int ncol, int len, int P, bool two_phase) {
-  RowsLayout R;
-  R.lw = (len + P - 1) / P;
-  R.lv = (ncol + P - 1) / P;
-  R.npairs = (ncol + 1) / 2;
-  R.kc = imax(1, imin(32, 2048 / imax(ncol, 1)));      // staged rows of V per chunk (<= 16 KB)
-  size_t o = 0;
-  auto take = [&](size_t bytes) { size_t r = o; o += (bytes + 15) & ~(size_t)15; return r; };
-  auto rnd16 = [](size_t bytes) { return (bytes + 15) & ~(size_t)15; };
-  R.wl = take((size_t)ncol * R.lw * 8);
-  R.vl = take((size_t)ncol * R.lv * 8);
-  R.nrm = take((size_t)ncol * 8);
-  R.pcw = take((size_t)R.npairs * 8);
-  R.psw = take((size_t)R.npairs * 8);
-  R.pf = take((size_t)R.npairs * 4);
-  R.gl = take((size_t)imax(R.npairs, ncol) * 8);
-  // shared region: exchange buffers | Newton-Schulz and X V staging
-  const size_t xch = rnd16((size_t)2 * R.npairs * P * 8) + rnd16((size_t)ncol * P * 8);
-  const size_t stg = two_phase ? rnd16((size_t)ncol * R.lv * 8) + rnd16((size_t)ncol * R.kc * 8) +
-                                     rnd16((size_t)R.lw * R.kc * 8)
-                               : 0;
-  const size_t base = take(xch > stg ? xch : stg);
-  R.xb = base;
-  R.nbuf = base + rnd16((size_t)2 * R.npairs * P * 8);
-  R.gb = base;
-  R.st = base + rnd16((size_t)ncol * R.lv * 8);
-  R.xs = R.st + rnd16((size_t)ncol * R.kc * 8);
-  R.sig = take((size_t)ncol * 8);
-  R.perm = take((size_t)ncol * 4);
-  R.tail = take((size_t)(ncol + 2) * 8);
-  R.total = o;
-  return R;
-}
-
 template <typename S>
 __device__ __forceinline__ S fmx(S a, S b, S c) {
   if constexpr (sizeof(S) == 8) return fma(a, b, c);
@@ -750,15 +704,6 @@ __device__ inline void rows_xv(const RowsLayout& R, unsigned char* wa, const T* 
   __syncthreads();
 }
 
-static constexpr int SW_WIDE = -3;
-// Centre matrices whose sweeps the leader runs alone, as a cluster of one: the exchanges of a
-// round (~3 k of its 9 k cycles) cost more than the other CTAs' FP64 units bring for a
-// few columns, and below ~16 columns the refinement of FP64 data costs more than
-// the sweeps.  Ten channel steps (16^3, FP64): 62.2 -> 56.6 ms on average (58.7 with cluster
-// sweeps throughout), with 12 columns 57.9, 24 as 16, 32 worse for the roundings.  FP32 data
-// are refined from RF_MIN columns on (16 columns alone: 128^3 sums 55 -> 61 ms).
-static constexpr int SOLO_LEN = 128;
-template <typename T> struct Solo { static constexpr int cols = sizeof(T) == 8 ? 16 : RF_MIN - 1; };
 // FP64 one-sided Jacobi SVD of the centre matrix C (m x n, T, global) with the
 // rows of the Jacobi matrices split over the CTAs of the cluster and held in
 // shared memory.  X = the columns of C (n <= m) or of C^T, scaled by scl;
@@ -773,10 +718,10 @@ template <typename T> struct Solo { static constexpr int cols = sizeof(T) == 8 ?
 //   the FP64 sweeps run only where it could not finish, from the V it reached;
 // SW_WIDE: the same with FP32 sweeps over the cluster, V along (jacobi_wide), where X
 //   does not fit one CTA's registers;
-// -1 (FP32 data beyond that too): the leader's V0 is in the job's scratch;
+// SW_SCRATCH (FP32 data beyond that too): the leader's V0 is in the job's scratch;
 //   one FP64 Newton-Schulz step, spread over the CTAs by blocks of columns, makes it
 //   orthogonal to ~1e-12, W = X V is formed in FP64 and the FP64 sweeps finish;
-// -2, and FP64 data: FP64 sweeps from W = X, V = I.
+// SW_PLAIN: FP64 sweeps from W = X, V = I.
 // Column norms are recomputed exactly at the start of every sweep and at the end.
 // Every CTA then finds the same singular values, order and kept rank (the rank rule
 // of Eq.
@@ -799,7 +744,7 @@ __device__ __noinline__ int svd64_rows(ClusterCtx& cc, const RoundJob& J, int L,
   T* out = (T*)J.dst.base + core_offset(L, J.dst.cap, k);
   const int ncol = imin(m, n), len = imax(m, n);
   const bool trans = (n <= m);
-  const RowsLayout R = rows_layout(ncol, len, cc.P, two_phase);
+  const RowsLayout R = rows_layout(ncol, len, cc.P, rows_stage(sizeof(T), sw32));
   double* Wl = (double*)(wa + R.wl);
   double* Vl = (double*)(wa + R.vl);
   double* nrm = (double*)(wa + R.nrm);
@@ -906,7 +851,7 @@ __device__ __noinline__ int svd64_rows(ClusterCtx& cc, const RoundJob& J, int L,
     }
     cl_sync(cc);                                  // the staging space is the exchange buffers' again
     if (phase_acc && threadIdx.x == 0) phase_acc[PH_XV] += (double)(clock64() - t1);
-  } else if (two_phase && sw32 == -1) {
+  } else if (two_phase && sw32 == SW_SCRATCH) {
     const long long t0 = clock64();
     float* V0 = (float*)(scr + J.lay.jv_off);
     const int ld0 = jacobi_ld<float>(ncol);
@@ -1072,25 +1017,23 @@ __device__ __noinline__ int svd64_site(const RoundJob& J, int L, int k, const T*
   const double scl = sh.tau[1];
   const int maxsw = J.max_sweeps > 0 ? J.max_sweeps : 60;
   // few columns: the sweeps of this CTA alone (a cluster of one)
-  const bool solo = cc.P > 1 && ncol <= Solo<T>::cols && len <= SOLO_LEN;
+  const Svd64Path path = cc.P > 1 ? svd64_path(ncol, len, cc.P, sizeof(T), J.refine) : Svd64Path{};
+  const bool solo = path.solo;
   ClusterCtx one = cc;
   one.P = 1;
   one.rank = 0;
-  if (solo || (!in_smem && cc.P > 1 && rows_layout(ncol, len, cc.P, sizeof(T) == 4).total <= (size_t)SM_WORK)) {
+  if (solo || path.rows) {
     // rows of the Jacobi matrices spread over the cluster, in shared memory
     pc.lap(PH_SVD_OUT);
     int sw32 = 0;
     bool logged = false;
-    const bool plain = solo || ncol < RF_MIN;     // FP64 sweeps from V = I
-    const bool refine = J.refine && rf_bytes(ncol, len, cc.P) <= (size_t)SM_WORK;
-    const bool wide = refine && !jacobi_reg_fits(ncol, len) && jacobi_wide_fits(ncol, len, cc.P);
-    if (!plain && !wide && (sizeof(T) == 4 || J.refine)) {
+    if (path.reg || (sizeof(T) == 4 && !path.plain && !path.wide)) {
       // FP32 sweeps on X by this CTA alone (its own stopping rule, a
       // sweep limit, convergence not required).  In registers where X fits: W only,
       // the rotations logged for the cluster to form V0 (a row of V0 per half-warp,
       // ~1/16 of the sweeps' time on 16 CTAs, where carrying V along would double
       // the sweeps' work)
-      if (refine && jacobi_reg_fits(ncol, len)) {
+      if (path.reg) {
         float* Wf = (float*)work;
         const int ldw32 = jacobi_reg_ld(len), ncp = jacobi_reg_cols(ncol);
         for (int idx = threadIdx.x; idx < ncp * ldw32; idx += blockDim.x) {
@@ -1125,7 +1068,7 @@ __device__ __noinline__ int svd64_site(const RoundJob& J, int L, int k, const T*
       if (threadIdx.x == 0) pc.acc[PH_SWEEPS32] += sw32;
       pc.lap(PH_J32);
     }
-    const int start = wide ? SW_WIDE : logged ? sw32 : plain ? -2 : -1;
+    const int start = path.wide ? SW_WIDE : logged ? sw32 : path.plain || sizeof(T) == 8 ? SW_PLAIN : SW_SCRATCH;
     if (!solo) cl_command(cc, 2, ncol, len, maxsw, m, n, k, delta, scl, start);
     int sw = 0;
     bool noconv = false;
@@ -1133,7 +1076,7 @@ __device__ __noinline__ int svd64_site(const RoundJob& J, int L, int k, const T*
     const int r = svd64_rows<T>(solo ? one : cc, J, L, k, m, n, scl, delta, maxsw, start, &sw, &noconv, &xfl, pc.on ? pc.acc : nullptr);
     pc.lap(PH_JACOBI);
     if (threadIdx.x == 0) { pc.acc[PH_SVD64_FLOPS] += svd_flops(m, n); pc.acc[PH_SVD64_EXEC] += xfl; }
-    const RowsLayout R = rows_layout(ncol, len, solo ? 1 : cc.P, sizeof(T) == 4);
+    const RowsLayout R = rows_layout(ncol, len, solo ? 1 : cc.P, rows_stage(sizeof(T), start));
     const unsigned char* wa = (const unsigned char*)work;
     const double* sig = (const double*)(wa + R.sig);
     const int* perm = (const int*)(wa + R.perm);
