@@ -236,8 +236,8 @@ int round_cluster_resident(int P);
 // doubles of scratch it takes), its scratch, and the eigenvectors of one (round.cu)
 size_t plan_gram_eig(RoundJob& j, int mmax);
 void place_gram_eig(RoundJob& j, double* scratch);
-void launch_gram_eig(const RoundJob* d_job, const double* G, int m, double* U, int chi, double delta2, int ncols_cap,
-                     int* r_out, int* status, cudaStream_t st);
+cudaError_t launch_gram_eig(const RoundJob* d_job, const double* G, int m, double* U, int chi, double delta2,
+                            int ncols_cap, int* r_out, int* status, cudaStream_t st);
 // increments the device step counter read by the rank model
 void launch_learn_tick(int* d_step, cudaStream_t st);
 

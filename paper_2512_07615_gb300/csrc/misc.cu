@@ -398,11 +398,13 @@ int tt_svd_dense(const T* d_dense, int n, T* d_dst, int* d_dst_ranks, int dst_ca
     const int P = (int)std::min<size_t>((size_t)Pg, nch);
     gram_part_kernel<<<P, 256, (size_t)m * kc * sizeof(double), st>>>(M, m, ncols, kc, P, gpart);
     gram_reduce_kernel<<<152, 256, 0, st>>>(gpart, P, (size_t)m * m, G);
-    launch_gram_eig(d_job, G, m, U, imin(chi_max, dst_cap), delta * delta,
-                    (int)(ncols < (size_t)1024 ? ncols : (size_t)1024), d_r, d_status, st);
+    // a launch that failed leaves d_r and U unwritten, and the stream's status does not tell
+    cudaError_t e = launch_gram_eig(d_job, G, m, U, imin(chi_max, dst_cap), delta * delta,
+                                    (int)(ncols < (size_t)1024 ? ncols : (size_t)1024), d_r, d_status, st);
     int h_r = 0;
-    cudaMemcpyAsync(&h_r, d_r, sizeof(int), cudaMemcpyDeviceToHost, st);
-    cudaError_t e = cudaStreamSynchronize(st);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(&h_r, d_r, sizeof(int), cudaMemcpyDeviceToHost, st);
+    const cudaError_t es = cudaStreamSynchronize(st);
+    if (e == cudaSuccess) e = es;
     if (e != cudaSuccess) { cleanup(); return cuda_fail(e, "tt_svd_dense"); }
     const int rn = h_r;
     if (rn > bond_cap(L, dst_cap, k + 1)) { cleanup(); return TNLBM_E_CAPACITY; }

@@ -2027,17 +2027,18 @@ size_t plan_gram_eig(RoundJob& j, int mmax) {
   return j.lay.total = off;
 }
 
-// scratch: plan_gram_eig's bytes in doubles; h_job (on the host) stays until d_job is written.
+// scratch: the doubles that plan_gram_eig returned.  j is copied to the device after this.
 void place_gram_eig(RoundJob& j, double* scratch) {
   j.scratch = scratch;
   j.dst.base = scratch + j.lay.q_off[0];
   j.dst.ranks = (int*)(scratch + j.lay.q_off[1]);
 }
 
-void launch_gram_eig(const RoundJob* d_job, const double* G, int m, double* U, int chi, double delta2, int ncols_cap,
-                     int* r_out, int* status, cudaStream_t st) {
-  cudaFuncSetAttribute(gram_eig_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)round_smem_bytes());
-  cudaFuncSetAttribute(gram_eig_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+cudaError_t launch_gram_eig(const RoundJob* d_job, const double* G, int m, double* U, int chi, double delta2,
+                            int ncols_cap, int* r_out, int* status, cudaStream_t st) {
+  cudaError_t e = cudaFuncSetAttribute(gram_eig_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)round_smem_bytes());
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(gram_eig_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+  if (e != cudaSuccess) return e;
   cudaLaunchConfig_t cfg = {};
   cfg.blockDim = dim3(RT, 1, 1);
   cfg.dynamicSmemBytes = round_smem_bytes();
@@ -2060,7 +2061,7 @@ void launch_gram_eig(const RoundJob* d_job, const double* G, int m, double* U, i
   }
   at[0].val.clusterDim.x = P;
   cfg.gridDim = dim3(P, 1, 1);
-  cudaLaunchKernelEx(&cfg, gram_eig_kernel, d_job, G, m, U, chi, delta2, ncols_cap, r_out, status);
+  return cudaLaunchKernelEx(&cfg, gram_eig_kernel, d_job, G, m, U, chi, delta2, ncols_cap, r_out, status);
 }
 
 template <typename T>
