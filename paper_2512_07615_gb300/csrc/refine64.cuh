@@ -408,9 +408,13 @@ __device__ __noinline__ int rf_refine(ClusterCtx& cc, RefineMem<N>& m, int n, in
 // not below ~1e-16 s_0 / s_j (FP64) whatever V is, while Jacobi rotations of W would keep them
 // small.  Where the directions of W are the orthonormal result (X is C^T), the columns are
 // made orthogonal: from every column go its parts along the larger ones (first order, at most
-// four times; the larger ones are left as they are), which changes W by those cosines
-// times s_j, its own rounding.  low: squared norms (relative to the largest) of columns
-// that are all rounding; they are left out.  False: this CTA has given up.
+// four times; the larger ones are left as they are), W <- W (I + F).  V takes the inverse,
+// V <- V (I - F^T), so that W V^T, the product of the result, stays X: those parts are up to
+// 1e-16 s_0 each, and all into the same few large directions (left in W alone they took FP64
+// sums of 64^3 populations from 1e-14 to 4e-14 off in single cells).  V is then orthonormal to
+// |F| ~ 1e-16 s_0 / s_i only, which its caller multiplies by s_i.  low: squared norms
+// (relative to the largest) of columns that are all rounding; they are left out.  False:
+// this CTA has given up.
 template <typename N>
 __device__ __noinline__ bool rf_polish(ClusterCtx& cc, RefineMem<N>& m, int n, int len, float low, float tol2, int at,
                                        int room) {
@@ -446,13 +450,23 @@ __device__ __noinline__ bool rf_polish(ClusterCtx& cc, RefineMem<N>& m, int n, i
                    if (c2 > 0.25f * tol2 && (si > sc || (si == sc && i < c))) f = -g / si;
                  }
                  F[(size_t)j * n + i] = f;
+                 __stcg(m.J + (size_t)c * m.ldj + i, f);
                });
     float s[4] = {rf_block_max(mx, s_red), 0.f, 0.f, 0.f};
     if (!rf_meet_max(cc, m, s)) return false;
     if (s[0] <= tol2) break;
     rf_gemm<float>(len, vi, n, [&](int k, int i) { return rf_f(__ldcg(m.W + (size_t)k * m.ldw + i)); }, false, F, n, (float*)st, rm,
                    [&](int i, int j, float v) { blk[(size_t)j * len + i] = rf_add(blk[(size_t)j * len + i], v); });
-    if (!cl_sync(cc)) return false;                        // W has been read everywhere
+    // V2(:, own) = V(:, own) - V F^T(:, own)
+    for (int k = threadIdx.x >> 5; k < n; k += blockDim.x >> 5)
+      for (int j = threadIdx.x & 31; j < vi; j += 32) F[(size_t)j * n + k] = __ldcg(m.J + (size_t)k * m.ldj + v0 + j);
+    rf_gemm<float>(n, vi, n, [&](int k, int i) { return rf_f(__ldcg(m.V + (size_t)k * m.ldv + i)); }, false, F, n, (float*)st, rm,
+                   [&](int i, int j, float v) {
+                     const size_t at = (size_t)(v0 + j) * m.ldv + i;
+                     __stcg(m.V2 + at, rf_add(__ldcg(m.V + at), -v));
+                   });
+    if (!cl_sync(cc)) return false;                        // W, V and F have been read everywhere
+    { N* t = m.V; m.V = m.V2; m.V2 = t; }
     for (int j = threadIdx.x >> 5; j < vi; j += blockDim.x >> 5)
       for (int k = threadIdx.x & 31; k < len; k += 32) __stcg(m.W + (size_t)(v0 + j) * m.ldw + k, blk[(size_t)j * len + k]);
     if (!cl_sync(cc)) return false;

@@ -1,0 +1,61 @@
+"""FP64 roundings whose centre SVDs are refined, against 64-bit fields: what the refinement does to
+W and V may cost rounding only."""
+import numpy as np
+import pytest
+
+from oracle import mps as M, quantics as q
+
+pytestmark = pytest.mark.gpu
+U = 2.0 ** -53
+
+
+@pytest.fixture(scope="module")
+def tl():
+    import torch
+    if not torch.cuda.is_available():
+        pytest.skip("no GPU")
+    import __graft_entry__
+    __graft_entry__.build()
+    from paper_2512_07615_gb300 import tnlbm as T
+    return T
+
+
+def train(L, r, rng):
+    """A random tensor train of bond r with orthonormal rows, entries of order one."""
+    b = [min(r, 2 ** k, 2 ** (L - k)) for k in range(L + 1)]
+    return [np.sqrt(2.0) * np.linalg.qr(rng.standard_normal((2 * b[k + 1], b[k])))[0].T.reshape(b[k], 2, b[k + 1])
+            for k in range(L)]
+
+
+def population(L, bond, seed):
+    """A constant and trains of bond four whose amplitudes fall over eight decades, as a sum
+    of blocks (bonds of at most 2^k and 2^(L - k) at the ends)."""
+    rng = np.random.default_rng(seed)
+    parts = (bond - 1) // 4
+    terms = [(1.0 / 18.0, M.ones(L))] + [(1e-3 / 18.0 * 10.0 ** (-8.0 * i / (parts - 1)), train(L, 4, rng)) for i in range(parts)]
+    c = M.lincomb(terms)
+    for k in range(L):
+        if 2 ** (k + 1) <= c[k].shape[2]:
+            m = c[k].reshape(2 ** (k + 1), -1)
+            c[k], c[k + 1] = np.eye(len(m)).reshape(-1, 2, len(m)), np.einsum("ab,bsc->asc", m, c[k + 1])
+    for k in range(L - 1, 0, -1):
+        if 2 ** (L - k) <= c[k].shape[0]:
+            m = c[k].reshape(c[k].shape[0], -1)
+            c[k], c[k - 1] = np.eye(m.shape[1]).reshape(m.shape[1], 2, -1), np.einsum("asb,bc->asc", c[k - 1], m)
+    return c
+
+
+@pytest.mark.parametrize("axis", [0, 1, 2])
+def test_untruncated_shift(tl, axis):
+    """A shift of a 64^3 population without truncation: centre matrices of 90 x 180 whose
+    singular values go down to rounding.  Four products a site (R W, QR, X V, Q U S) of
+    sums of at most 180 terms leave sqrt(4 L 180) u of the largest value; the largest of 2^18
+    cells is allowed half as much again."""
+    L, bond = 18, 45
+    x = population(L, bond, 11)
+    X = tl.DeviceMps.from_cores(x, bond, tl.nat.FP64)
+    dst = tl.DeviceMps(L, 2 * bond, tl.nat.FP64)
+    tl.lincomb_round([[tl.shift(X, axis, 1)]], [dst], 2 * bond, 1e-16)
+    got = q.decode(M.to_tensor([np.asarray(c) for c in dst.cores()]))
+    ref = np.roll(q.decode(M.to_tensor(x)), -1, axis)
+    assert np.abs(got - ref).max() <= 1.5 * np.sqrt(4 * L * 4 * bond) * U * np.abs(ref).max()
