@@ -447,7 +447,7 @@ struct Builder {
 // Options every rounding job of a simulation carries.
 static void set_round_options(const tnlbm_sim* s, RoundJob& rj) {
   rj.svd64 = prec_svd64(s->prec) ? 1 : 0;
-  rj.refine = (rj.svd64 || s->prec == TNLBM_FP64) ? 1 : 0;
+  rj.refine = (rj.svd64 || s->prec == TNLBM_FP64) ? REFINE_OWN : REFINE_OFF;
   rj.max_sweeps = s->cfg.jacobi_max_sweeps;
   rj.wait_ns = s->cfg.wait_limit_ns;
 }
@@ -1540,7 +1540,7 @@ static int lincomb_impl(int n_bits, int batch, int nterms, const tnlbm_term* ter
     RoundJob& j = jobs[b];
     j = RoundJob{};
     j.svd64 = svd64;
-    j.refine = !materialize && (svd64 || sizeof(T) == 8) ? 1 : 0;
+    j.refine = !materialize && (svd64 || sizeof(T) == 8) ? REFINE_OWN : REFINE_OFF;
     j.nterms = nterms;
     j.chi = chi;
     j.eps = eps;

@@ -136,6 +136,9 @@ struct LearnCtx {
   int* counters;              // [0] randomized accepted, [1] fell back, [2] full SVDs
 };
 
+// FP64 SVDs of a job: not refined; to the scale of every column (FP64 data); to that of the largest
+enum : int { REFINE_OFF = 0, REFINE_OWN = 1, REFINE_TOP = 2 };
+
 struct RoundJob {
   int nterms;
   int chi;
@@ -157,7 +160,7 @@ struct RoundJob {
   int L, n_bits;              // chain length and bits per axis of this job, or 0 = launch's
   double* discard;            // accumulator of squared discarded tails (device), or null
   int svd64;                  // 1: centre SVDs in FP64 on FP32 data (precision TNLBM_MIXED)
-  int refine;                 // 1: scratch for refined FP64 SVDs (launches with clusters)
+  int refine;                 // REFINE_*: scratch for refined FP64 SVDs (launches with clusters)
   int max_sweeps;             // Jacobi sweep limit (0 = 60)
   long long wait_ns;          // limit of every cross-CTA wait in ns (0 = 5 s)
 };

@@ -243,19 +243,22 @@ enum : int { RF_DONE = 0, RF_SWEEPS = 1, RF_DEAD = 2 };
 // consecutive in memory.  ties: pairs of equal singular values may keep their
 // cosine.  jacobi(): one FP32 Jacobi of W by the leader with its rotations formed in
 // m.J over the cluster (false: not available).  A pair is orthogonal if its squared
-// cosine is at most tol2, or if turning it would move no more than tmin s_0 of its larger
-// column (|t| s_i <= tmin s_0): W = X V carries the rounding of s_0 in every column, so
-// small columns turn by such angles for ever, and a graded spectrum went through all steps
-// and the FP64 sweeps.  With the larger column's own scale in place of s_0: 128^3 sums at
-// bond 64, mixed, 57 ms for 40; 256^3 at bond 128, 232 for 142; FP64 64^3 sums at bond 45, 51 for
-// 48, with an error of 2.8e-15 where nothing is discarded (3.2e-15 before, 2.1e-15 of the
-// sweeps; tmin = 1e-15 would give 40 ms and 1.1e-14).
+// cosine is at most tol2, or if its tangent t is small enough to be W's rounding:
+// own_scale: |t| <= tmin, to the columns' own scale; else |t| s_i <= tmin s_0 for its larger
+// column.  W = X V carries a rounding of s_0, which turns small columns by more than
+// their own scale, but the rows of a centre matrix are graded as its singular values are, and
+// then small directions are as well determined as large ones: FP64 roundings need the own
+// scale (with s_0, 1e-12 in the start of a porous 128^3 flow grew to 4.6e-7 in three steps at
+// bond 64, where the FP64 sweeps and the own scale have 6.0e-9 and 2.9e-9).  FP32 data hold nothing
+// below s_0 tmin: 128^3 sums at bond 64, mixed, 40 ms, with the own scale 57; 256^3 at bond 128,
+// 142 and 232.  FP64 pays 64^3 sums at bond 45 47.9 -> 49.4 ms, 32^3 walls 13.1 -> 14.5.  Eigenproblems of
+// Gram matrices (REFINE_TOP) hold nothing below s_0's rounding either.
 // small: the largest |E| whose square, and whose FP32 product's error, are below
 // what V has to be accurate to; ready: the |R| from which a Jacobi of W pays; none:
 // squared norms (relative to the largest) of columns whose pairs carry nothing.
 template <typename N, typename FX, typename FJ>
 __device__ __noinline__ int rf_refine(ClusterCtx& cc, RefineMem<N>& m, int n, int len, bool go_on, FX x, bool kfast,
-                                      bool ties, float tol2, float tmin, float small, float ready, float none, int at, int room,
+                                      bool ties, float tol2, float tmin, bool own_scale, float small, float ready, float none, int at, int room,
                                       FJ jacobi) {
   extern __shared__ __align__(16) unsigned char smem[];
   unsigned char* wa = smem + at;                           // the work area (`room` bytes), known to be shared memory
@@ -331,7 +334,7 @@ __device__ __noinline__ int rf_refine(ClusterCtx& cc, RefineMem<N>& m, int n, in
                      if (c2 > tol2) {
                        const float z = rf_diff(nr[c], nr[i]) / (2.f * g), az = fabsf(z);
                        const float t = copysignf(az > 1e15f ? 0.5f / az : 1.f / (az + sqrtf(fmaf(z, z, 1.f))), z);
-                       if (t * t * sb <= tmin2) {
+                       if (own_scale ? fabsf(t) <= tmin : t * t * sb <= tmin2) {
                          // nothing: W's own rounding
                        } else if (fabsf(t) <= 0.1f) {
                          e += t;

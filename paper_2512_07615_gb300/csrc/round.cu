@@ -828,10 +828,11 @@ __device__ __noinline__ int svd64_rows(ClusterCtx& cc, const RoundJob& J, int L,
     };
     const T tscl = (T)scl;                        // exact: a power of two
     auto xn = [&](int i, int kk) -> N { return rf_make<N>(tscl * __ldcg(trans ? C + (size_t)i * n + kk : C + (size_t)kk * n + i)); };
+    const bool own = !two_phase && J.refine != REFINE_TOP;
     // the sums of FP32 data carry 48 bits
     const float tol2r = (two_phase ? 256.f : 1.f) * (float)(tol64 * tol64);
     state = rf_refine<N>(cc, rm, ncol, len, sw32 < maxsw, xn, trans, trans, tol2r,
-                         two_phase ? 2e-13f : 1e-16f, two_phase ? 2e-6f : 2e-9f, two_phase ? 1e-11f : 1e-14f,
+                         two_phase ? 2e-13f : own ? 4e-16f : 1e-16f, own, two_phase ? 2e-6f : 2e-9f, two_phase ? 1e-11f : 1e-14f,
                          two_phase ? 1e-22f : 1e-28f, SM_SMALL, SM_WORK, jacobi);
     if (state == RF_DONE && !trans && !rf_polish<N>(cc, rm, ncol, len, low, tol2r, SM_SMALL, SM_WORK)) state = RF_DEAD;
     if (phase_acc && threadIdx.x == 0) phase_acc[PH_NS] += (double)(clock64() - t0);
@@ -2009,7 +2010,7 @@ size_t plan_gram_eig(RoundJob& j, int mmax) {
   j.L = 3;
   j.n_bits = 1;
   j.chi = mmax;
-  j.refine = 1;
+  j.refine = REFINE_TOP;
   j.dst.cap = mmax;
   size_t off = 0;
   auto al = [&](size_t n) { const size_t o = off; off += (n + 31) & ~(size_t)31; return o; };

@@ -59,3 +59,44 @@ def test_untruncated_shift(tl, axis):
     got = q.decode(M.to_tensor([np.asarray(c) for c in dst.cores()]))
     ref = np.roll(q.decode(M.to_tensor(x)), -1, axis)
     assert np.abs(got - ref).max() <= 1.5 * np.sqrt(4 * L * 4 * bond) * U * np.abs(ref).max()
+
+
+def isometries(L, k, sig, r1, rng):
+    """Cores of an MPS that is an isometry on both sides of bond k, the singular values sig
+    there and a bond of r1 to its right; and the 2^(L-k) rows of their right vectors."""
+    r = len(sig)
+    bonds = [min(2 ** j, r) for j in range(k + 1)] + [min(2 ** (L - j), r1) for j in range(k + 1, L + 1)]
+    orth = lambda m, n: np.linalg.qr(rng.standard_normal((m, n)))[0]
+    cores = [orth(bonds[j] * 2, bonds[j + 1]).reshape(bonds[j], 2, bonds[j + 1]) for j in range(k)]
+    cores += [orth(2 * bonds[j + 1], bonds[j]).T.reshape(bonds[j], 2, bonds[j + 1]) for j in range(k, L)]
+    rows = right_rows(cores[k:])
+    cores[k] = cores[k] * sig[:, None, None]
+    return cores, rows
+
+
+def right_rows(cores):
+    right = np.ones((1, 1))
+    for c in reversed(cores):
+        right = np.einsum("asb,bq->asq", c, right).reshape(c.shape[0], -1)
+    return right
+
+
+# r columns of 2 r1 entries: as many rows as columns (V is the result) and fewer (W is)
+@pytest.mark.parametrize("r,r1,chi", [(120, 60, 60), (100, 62, 62), (64, 32, 32), (100, 50, 50)])
+@pytest.mark.parametrize("seed", [0, 1, 2])
+def test_small_directions(tl, r, r1, chi, seed):
+    """Ten decades of singular values cut at chi: the kept directions against the discarded ones.
+    The rows of the centre matrix are graded as the singular values are, so its
+    rounding turns a pair by ~u sqrt(n) (1 / q - q)^-1, q the ratio of neighbours, and the
+    sweeps' own tolerance, 16 * 2 u sqrt(n) of a pair's cosine, by as much as that."""
+    L, k = 15, 7
+    rng = np.random.default_rng(100 * r + seed)
+    sig = 10.0 ** (-10.0 * np.arange(r) / (r - 1))
+    cores, rows = isometries(L, k, sig, r1, rng)
+    X = tl.DeviceMps.from_cores(cores, r, tl.nat.FP64)
+    dst = tl.DeviceMps(L, chi, tl.nat.FP64)
+    tl.lincomb_round([[tl.plain(X)]], [dst], chi, 1e-14)
+    got = right_rows([np.asarray(c) for c in dst.cores()][k:])
+    assert got.shape[0] == chi
+    ratio = sig[1] / sig[0]
+    assert np.abs(got @ rows[chi:].T).max() <= 32 * U * np.sqrt(2 * r1) / (1 / ratio - ratio)
