@@ -126,17 +126,19 @@ __device__ __forceinline__ void qr_reg_update(float* V, int mr, float* X, int ld
     float* x = X + c;
 #pragma unroll 4
     for (int r = r0; r < r1; ++r) {
-      float s = x[(size_t)r * ld];
+      // the change first: taken from X term by term it would round sixteen times at X's size
+      // (directions of mixed roundings 8-16 % further off)
+      float s = 0.f;
       const float4* v = (const float4*)(V + (size_t)r * 16);
 #pragma unroll
       for (int i = 0; i < 4; ++i) {
         const float4 w = v[i];
-        s = fmaf(-w.x, a[4 * i], s);
-        s = fmaf(-w.y, a[4 * i + 1], s);
-        s = fmaf(-w.z, a[4 * i + 2], s);
-        s = fmaf(-w.w, a[4 * i + 3], s);
+        s = fmaf(w.x, a[4 * i], s);
+        s = fmaf(w.y, a[4 * i + 1], s);
+        s = fmaf(w.z, a[4 * i + 2], s);
+        s = fmaf(w.w, a[4 * i + 3], s);
       }
-      x[(size_t)r * ld] = s;
+      x[(size_t)r * ld] -= s;
     }
   }
   __syncthreads();
