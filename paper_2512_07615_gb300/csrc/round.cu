@@ -388,7 +388,7 @@ __device__ __forceinline__ void renorm64(float cf, float sf, double& c, double& 
 // orthogonal to FP64 rounding: for |t| < 2^-14 by the series c = 1 - t^2/2,
 // s = t c; else the FP32 (c, s) renormalised in FP64 (renorm64).  The new
 // norms are al - t g and be + t g (exact for the exact root; recomputed every
-// sweep); rel2 = g^2 / (al be) for the stopping rule.
+// sweep); rel2 = g^2 / (al be) and tan = |t| for the stopping rule.
 // A warp's FP64 instruction takes 64 cycles of its scheduler (0.5 lanes a clock), and a
 // round waits for this chain: 30 of them took 4 k of a round's 9 k cycles.  So where al, be
 // and g are within 2^+-100 and al, be within 2^100 of each other, the test and the quotient
@@ -403,7 +403,7 @@ __device__ __forceinline__ double widen_bits(float x) {     // a normal number
   return __hiloint2double((int)((u & 0x80000000u) | (((u & 0x7fffffffu) >> 3) + 0x38000000u)), (int)(u << 29));
 }
 __device__ __forceinline__ bool rows_angle(double al, double be, double g, double tol2, double& cw, double& sw,
-                                           double& na, double& nb, float& rel2) {
+                                           double& na, double& nb, float& rel2, float& tan) {
   const int xa = __double2hiint(al) >> 20, xb = __double2hiint(be) >> 20, xg = (__double2hiint(g) >> 20) & 0x7ff;
   if (xa > 923 && xa < 1123 && xb > 923 && xb < 1123 && xg > 923 && xg < 1123 && xa - xb < 100 && xb - xa < 100) {
     const float gf = narrow_bits(g);
@@ -413,6 +413,7 @@ __device__ __forceinline__ bool rows_angle(double al, double be, double g, doubl
     const float z = (float)(be - al) / (2.f * gf), az = fabsf(z);
     const float tf = copysignf(az > 1e18f ? 0.5f / az : 1.f / (az + sqrtf(fmaf(z, z, 1.f))), z);
     const double t = widen_bits(tf);                        // at least 2^-100: normal
+    tan = fabsf(tf);
     if (fabsf(tf) < 6.1035156e-05f) {
       cw = fma(-0.5 * t, t, 1.0);                           // c^2 + s^2 = 1 - 3 t^4 / 4 + ...
       sw = t * cw;
@@ -449,6 +450,7 @@ __device__ __forceinline__ bool rows_angle(double al, double be, double g, doubl
     tf = copysignf(1.f / (fabsf(z) + sqrtf(fmaf(z, z, 1.f))), z);
     t = (double)tf;
   }
+  tan = fabsf((float)t);
   if (tiny) {
     cw = 1.0;                                           // 1 + t^2 rounds to 1 for |t| < 1e-18
     sw = t;
@@ -470,13 +472,14 @@ __device__ __forceinline__ bool rows_angle(double al, double be, double g, doubl
 // rows of W and V; nrot counts rotations.  Per round: each CTA's parts of the
 // pair inner products go to every CTA, four lanes per pair add them in rank
 // order, lane 0 takes the angle, and every CTA rotates its rows of W and V.
-// Stopping rule: a sweep that rotates nothing (every pair within the
-// tolerance), or a sweep whose largest relative inner product
-// g^2 / (al be) was below (5e-9)^2 -- Jacobi converges quadratically,
-// so its rotations leave every pair below ~(5e-9)^2 ncol plus the FP32 angle's
-// residual 1.2e-7 x 5e-9, under the tolerance 16 eps_64 sqrt(len) >= 5e-15,
-// and the confirming sweep is skipped.  Every CTA sees the same values, so
-// every CTA stops at the same sweep.  Returns the sweeps used; *converged
+// Stopping rule: a sweep that rotates nothing (every pair within the tolerance), or a
+// sweep whose cosines c and tangents t were small: c below 5e-9 and the largest c times the
+// largest t below a tenth of the tolerance.  A rotation turns t c of its columns' cosines
+// with others onto one another, so that is what a sweep leaves (and the FP32 angle's residual
+// 1.2e-7 x 5e-9, under the tolerance 16 eps_64 sqrt(len) >= 5e-15), and the confirming
+// sweep is skipped.  Columns of close singular values turn far on small cosines: with c alone,
+// eight of them 1e-9 apart kept cosines of up to 9e-10 after a refinement.  Every CTA sees the
+// same values, so every CTA stops at the same sweep.  Returns the sweeps used; *converged
 // tells whether the rule was met within maxsw sweeps.
 template <typename S>
 __device__ __noinline__ int rows_sweeps(ClusterCtx& cc_, const RowsLayout& R_, unsigned char* wa, S* Wl, double* Vl, int ncol,
@@ -487,7 +490,7 @@ __device__ __noinline__ int rows_sweeps(ClusterCtx& cc_, const RowsLayout& R_, u
   // the exchanges that a round is made of
   ClusterCtx cc = cc_;
   const RowsLayout R = R_;
-  __shared__ float s_mrel[32];
+  __shared__ float s_mrel[32], s_mtan[32];
   RxClock rx(phase_acc);
   unsigned q = 0;                                  // rounds so far (exchange buffer parity)
   S* nrm = (S*)(wa + R.nrm);
@@ -519,7 +522,7 @@ __device__ __noinline__ int rows_sweeps(ClusterCtx& cc_, const RowsLayout& R_, u
     rows_norms<S>(cc, R, wa, Wl, ncol, li);
     rx.lap(PH_RX_NORM);
     int any = 0;
-    float mrel = 0.f;                              // largest g^2 / (al be) this thread rotated this sweep
+    float mrel = 0.f, mtan = 0.f;                  // largest g^2 / (al be) and |t| this thread rotated this sweep
     bool ok = rows_pair_dots<S>(cc, R, wa, Wl, xb + (size_t)(q & 1) * npairs * cc.P, 0, np, ncol, li, rx);
     for (int rnd = 0; rnd < np - 1 && ok; ++rnd, ++q) {
       const S* xq = xb + (size_t)(q & 1) * npairs * cc.P;
@@ -544,9 +547,10 @@ __device__ __noinline__ int rows_sweeps(ClusterCtx& cc_, const RowsLayout& R_, u
         int go = 0;
         if (b < ncol) {
           S cw, sw, na, nb;
-          float rel2 = 0.f;
-          if (rows_angle(nrm[a], nrm[b], g, tol2, cw, sw, na, nb, rel2)) {
+          float rel2 = 0.f, tan = 0.f;
+          if (rows_angle(nrm[a], nrm[b], g, tol2, cw, sw, na, nb, rel2, tan)) {
             mrel = fmaxf(mrel, rel2);
+            mtan = fmaxf(mtan, tan);
             nrm[a] = na;
             nrm[b] = nb;
             pcw[p] = cw;
@@ -582,14 +586,17 @@ __device__ __noinline__ int rows_sweeps(ClusterCtx& cc_, const RowsLayout& R_, u
     }
     if (cc.dead) break;
     if (!any) { *converged = true; break; }
-    // the sweep's largest relative inner product (the same in every CTA)
-    for (int o = 16; o > 0; o >>= 1) mrel = fmaxf(mrel, __shfl_xor_sync(0xffffffffu, mrel, o));
-    if ((threadIdx.x & 31) == 0) s_mrel[threadIdx.x >> 5] = mrel;
+    // the sweep's largest cosine (squared) and tangent (the same in every CTA)
+    for (int o = 16; o > 0; o >>= 1) {
+      mrel = fmaxf(mrel, __shfl_xor_sync(0xffffffffu, mrel, o));
+      mtan = fmaxf(mtan, __shfl_xor_sync(0xffffffffu, mtan, o));
+    }
+    if ((threadIdx.x & 31) == 0) { s_mrel[threadIdx.x >> 5] = mrel; s_mtan[threadIdx.x >> 5] = mtan; }
     __syncthreads();
-    float m = 0.f;
-    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) m = fmaxf(m, s_mrel[w]);
+    float m = 0.f, mt = 0.f;
+    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) { m = fmaxf(m, s_mrel[w]); mt = fmaxf(mt, s_mtan[w]); }
     __syncthreads();
-    if (m < 2.5e-17f) { *converged = true; ++sweep; break; }
+    if (m < 2.5e-17f && sqrtf(m) * mt < 0.1f * sqrtf((float)tol2)) { *converged = true; ++sweep; break; }
   }
   if (phase_acc && threadIdx.x == 0) phase_acc[PH_ROUNDS64] += rounds;
   if (rounds_out) *rounds_out = rounds;

@@ -100,3 +100,33 @@ def test_small_directions(tl, r, r1, chi, seed):
     assert got.shape[0] == chi
     ratio = sig[1] / sig[0]
     assert np.abs(got @ rows[chi:].T).max() <= 32 * U * np.sqrt(2 * r1) / (1 / ratio - ratio)
+
+
+def close_values(tl, r, r1, chi, width, gap, seed):
+    """The largest part of a kept direction along a discarded one, where the cut at chi lies in the
+    middle of `width` singular values of relative distance gap."""
+    L, k = 15, 7
+    rng = np.random.default_rng(1000 * r + seed)
+    sig = 10.0 ** (-np.arange(r) / (r - 1))
+    sig[chi - width // 2:chi + width // 2] = sig[chi] * (1.0 - gap * np.arange(width))
+    cores, rows = isometries(L, k, sig, r1, rng)
+    mix = np.linalg.qr(rng.standard_normal((r, r)))[0]
+    cores[k] = np.einsum("ab,bsc->asc", mix, cores[k])
+    X = tl.DeviceMps.from_cores(cores, r, tl.nat.FP64)
+    dst = tl.DeviceMps(L, chi, tl.nat.FP64)
+    tl.lincomb_round([[tl.plain(X)]], [dst], chi, 1e-14)
+    got = right_rows([np.asarray(c) for c in dst.cores()][k:])
+    return np.abs(got @ rows[chi:].T).max()
+
+
+# The sweeps' tolerance of a pair's cosine, 16 * 2 u sqrt(n), and the centre matrix's rounding, four
+# products of sums of n terms at s_0 / s_chi <= 4, over the difference of the pair's squares:
+def close_bound(r1, gap):
+    return (32 + 4 * 4) * U * np.sqrt(2 * r1) / (2 * gap)
+
+
+# fewer rows than columns: the sweeps finish what the refinement leaves of close values
+@pytest.mark.parametrize("r,r1,chi", [(100, 62, 62), (60, 40, 40)])
+@pytest.mark.parametrize("seed", [0, 1, 2, 3])
+def test_sweeps_of_close_values(tl, r, r1, chi, seed):
+    assert close_values(tl, r, r1, chi, 8, 1e-9, seed) <= close_bound(r1, 1e-9)
