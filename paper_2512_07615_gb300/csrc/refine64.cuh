@@ -26,7 +26,8 @@
 // Pairs whose singular values agree to ~1e-5 (|t| large although the cosine is
 // below 1e-5) may keep their cosine: any basis of their span serves, since V stays
 // orthonormal, W = X V holds whatever the basis, and the discarded weight is the sum
-// of the discarded |w_j|^2.
+// of the discarded |w_j|^2.  Where the rank rule cuts between two such columns the basis
+// is the result: the caller lets the sweeps turn them (RF_TIE, RefineMem::tied).
 //
 // Work is split by columns: CTA c owns columns [c n / P, (c + 1) n / P) of V, W, S and
 // E, all in the job's scratch (L2); a cluster barrier separates the steps.  What is
@@ -46,6 +47,7 @@ namespace tn {
 static constexpr int RF_KC = 8;          // rows of k that at least are staged at a time
 static constexpr int RF_STEPS = 12;      // steps V <- V (I + E) at most
 static constexpr int RF_PASSES = 2;      // FP32 Jacobis of W at most
+static constexpr double RF_TIE = 2e-4;   // squared norms that agree to this may be of a pair that kept its cosine (|t| > 0.1, cosine <= 1e-5)
 static constexpr int RF_MIN = 6;         // columns from which it is taken: below, the few rounds of the sweeps cost less
 
 // A number of ~48 bits as the unevaluated sum of two floats (x = the rounded value),
@@ -210,6 +212,7 @@ struct RefineMem {
   float2* log;
   int ldv, ldw, ldj;
   int turn;                // meetings so far (the slots of stat alternate)
+  bool tied;               // pairs of equal singular values have kept their cosine
 };
 
 // All CTAs meet; the maxima over the cluster of the four values v (thread-uniform
@@ -360,6 +363,7 @@ __device__ __noinline__ int rf_refine(ClusterCtx& cc, RefineMem<N>& m, int n, in
     mt = (tied ? 1.f : 0.f) + (large ? 2.f : 0.f);
     float s[4] = {rf_block_max(mr, s_red), rf_block_max(mt, s_red), rf_block_max(mx, s_red), rf_block_max(dev, s_red)};
     if (!rf_meet_max(cc, m, s)) return RF_DEAD;
+    m.tied = s[1] == 1.f;
     bool only_r = !go_on;                                  // E = R / 2 only
     if (!only_r && s[1] >= 2.f) {
       if (passes >= RF_PASSES || step >= RF_STEPS) {

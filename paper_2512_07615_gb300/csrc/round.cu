@@ -765,6 +765,7 @@ __device__ __noinline__ int svd64_rows(ClusterCtx& cc, const RoundJob& J, int L,
   auto xat = [&](int i, int kk) -> double { return scl * (double)__ldcg(trans ? C + (size_t)i * n + kk : C + (size_t)kk * n + i); };
   const int ld1 = jacobi_ld<double>(ncol);
   int state = RF_SWEEPS;
+  bool tied = false;
   // squared norms relative to the largest below which a refined W is rounding only
   constexpr float low = two_phase ? 1e-22f : 1e-27f;
   if (sw32 >= 0 || sw32 == SW_WIDE) {
@@ -798,6 +799,7 @@ __device__ __noinline__ int svd64_rows(ClusterCtx& cc, const RoundJob& J, int L,
     rm.nrm = rm.V2 + (size_t)ncol * ld1;
     rm.log = (float2*)(scr + J.lay.log_off);
     rm.turn = 0;
+    rm.tied = false;
     if (wide) {
       sw32 = sweep_wide([&](int i, int j) { return (float)xat(i, j); });
       for (int idx = threadIdx.x; idx < ncol * vi; idx += blockDim.x)
@@ -841,6 +843,7 @@ __device__ __noinline__ int svd64_rows(ClusterCtx& cc, const RoundJob& J, int L,
     state = rf_refine<N>(cc, rm, ncol, len, sw32 < maxsw, xn, trans, trans, tol2r,
                          two_phase ? 2e-13f : own ? 4e-16f : 1e-16f, own, two_phase ? 2e-6f : 2e-9f, two_phase ? 1e-11f : 1e-14f,
                          two_phase ? 1e-22f : 1e-28f, SM_SMALL, SM_WORK, jacobi);
+    tied = rm.tied;
     if (state == RF_DONE && !trans && !rf_polish<N>(cc, rm, ncol, len, low, tol2r, SM_SMALL, SM_WORK)) state = RF_DEAD;
     if (phase_acc && threadIdx.x == 0) phase_acc[PH_NS] += (double)(clock64() - t0);
     const long long t1 = clock64();
@@ -937,11 +940,22 @@ __device__ __noinline__ int svd64_rows(ClusterCtx& cc, const RoundJob& J, int L,
       s_r = rr > bond_cap(L, J.dst.cap, k) ? 0 : rr;
     }
     __syncthreads();
-    // kept columns of W that are all rounding have no directions (a tolerance below the
-    // refinement's resolution): the sweeps orthogonalise them like any others
-    if (again || state != RF_DONE || trans || s_r < 1 || cc.dead) break;
+    // the sweeps finish like any others: kept columns of W that are all rounding and have no
+    // directions (a tolerance below the refinement's resolution), and pairs that kept their
+    // cosine on both sides of the cut (of a Gram matrix, whose cut is its caller's: anywhere
+    // above its rounding)
+    if (again || state != RF_DONE || s_r < 1 || cc.dead) break;
     const double s0 = sig[perm[0]], sl = sig[perm[s_r - 1]];
-    if (sl * sl > (double)low * s0 * s0) break;
+    bool more = !trans && sl * sl <= (double)low * s0 * s0;
+    if (tied) {
+      const bool top = J.refine == REFINE_TOP;
+      const double least = top ? 64.0 * 2.220446049250313e-16 * ncol * s0 : 0.0;
+      for (int p = top ? 1 : s_r; p < (top ? ncol : imin(s_r + 1, ncol)); ++p) {
+        const double a = sig[perm[p - 1]], b = sig[perm[p]];
+        more |= b > least && a * a - b * b <= RF_TIE * a * a;
+      }
+    }
+    if (!more) break;
     cl_sync(cc);                                  // the norms' slots have been read everywhere
     sw = rows_sweeps<double>(cc, R, wa, W, Vl, ncol, li, vi, maxsw, tol64 * tol64, &s_nrot, phase_acc, &conv, &rounds);
     *sweeps_out = sw;

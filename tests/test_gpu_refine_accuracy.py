@@ -130,3 +130,11 @@ def close_bound(r1, gap):
 @pytest.mark.parametrize("seed", [0, 1, 2, 3])
 def test_sweeps_of_close_values(tl, r, r1, chi, seed):
     assert close_values(tl, r, r1, chi, 8, 1e-9, seed) <= close_bound(r1, 1e-9)
+
+
+# as many rows as columns: the refinement may leave close values as they are, but not across the cut
+@pytest.mark.parametrize("r,r1,chi", [(64, 32, 32), (120, 60, 60)])
+@pytest.mark.parametrize("width,gap", [(2, 1e-7), (2, 1e-9), (8, 1e-9), (24, 1e-7)])
+@pytest.mark.parametrize("seed", [0, 1, 2, 3])
+def test_cut_between_close_values(tl, r, r1, chi, width, gap, seed):
+    assert close_values(tl, r, r1, chi, width, gap, seed) <= close_bound(r1, gap)
