@@ -414,16 +414,17 @@ __device__ __noinline__ int rf_refine(ClusterCtx& cc, RefineMem<N>& m, int n, in
 // W = X V carries the rounding of the whole X in its small columns, so their cosines are
 // not below ~1e-16 s_0 / s_j (FP64) whatever V is, while Jacobi rotations of W would keep them
 // small.  Where the directions of W are the orthonormal result (X is C^T), the columns are
-// made orthogonal: from every column go its parts along the larger ones (first order, at most
-// four times; the larger ones are left as they are), W <- W (I + F).  V takes the inverse,
+// made orthogonal: from every column go its parts along the larger ones (first order, the
+// larger ones are left as they are), W <- W (I + F).  V takes the inverse,
 // V <- V (I - F^T), so that W V^T, the product of the result, stays X: those parts are up to
 // 1e-16 s_0 each, and all into the same few large directions (left in W alone they took FP64
 // sums of 64^3 populations from 1e-14 to 4e-14 off in single cells).  V is then orthonormal to
-// |F| ~ 1e-16 s_0 / s_i only, which its caller multiplies by s_i.  low: squared norms
-// (relative to the largest) of columns that are all rounding; they are left out.  False:
-// this CTA has given up.
+// |F| ~ 1e-16 s_0 / s_i only, which its caller multiplies by s_i.  A round squares the sums of
+// a column's cosines and triples them: from 0.1 five rounds end below 1e-16.  Where a sum is
+// larger nothing is done.  low: squared norms (relative to the largest) of columns that are
+// all rounding; they are left out.  RF_DONE; RF_SWEEPS: the sweeps have to finish; or RF_DEAD.
 template <typename N>
-__device__ __noinline__ bool rf_polish(ClusterCtx& cc, RefineMem<N>& m, int n, int len, float low, float tol2, int at,
+__device__ __noinline__ int rf_polish(ClusterCtx& cc, RefineMem<N>& m, int n, int len, float low, float tol2, int at,
                                        int room) {
   extern __shared__ __align__(16) unsigned char smem[];
   unsigned char* wa = smem + at;
@@ -444,7 +445,7 @@ __device__ __noinline__ bool rf_polish(ClusterCtx& cc, RefineMem<N>& m, int n, i
   for (int i = threadIdx.x & 31; i < n; i += 32) nmax = fmaxf(nmax, rf_f(nr[i]));
   for (int o = 16; o > 0; o >>= 1) nmax = fmaxf(nmax, __shfl_xor_sync(0xffffffffu, nmax, o));
   const float least = low * nmax;
-  for (int it = 0; it < 4; ++it) {
+  for (int it = 0;; ++it) {
     float mx = 0.f;
     rf_gemm<N>(n, vi, len, [&](int k, int i) { return __ldcg(m.W + (size_t)i * m.ldw + k); }, true, blk, len, st, rm,
                [&](int i, int j, N s) {
@@ -459,9 +460,17 @@ __device__ __noinline__ bool rf_polish(ClusterCtx& cc, RefineMem<N>& m, int n, i
                  F[(size_t)j * n + i] = f;
                  __stcg(m.J + (size_t)c * m.ldj + i, f);
                });
-    float s[4] = {rf_block_max(mx, s_red), 0.f, 0.f, 0.f};
-    if (!rf_meet_max(cc, m, s)) return false;
-    if (s[0] <= tol2) break;
+    float sum = 0.f;                                       // of the cosines that F takes off a column
+    for (int j = threadIdx.x >> 5; j < vi; j += blockDim.x >> 5) {
+      float a = 0.f;
+      for (int i = threadIdx.x & 31; i < n; i += 32) a += fabsf(F[(size_t)j * n + i]) * sqrtf(rf_f(nr[i]));
+      for (int o = 16; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
+      sum = a > 0.f ? fmaxf(sum, a * rsqrtf(rf_f(nr[v0 + j]))) : sum;
+    }
+    float s[4] = {rf_block_max(mx, s_red), rf_block_max(sum, s_red), 0.f, 0.f};
+    if (!rf_meet_max(cc, m, s)) return RF_DEAD;
+    if (s[0] <= tol2) return RF_DONE;
+    if (s[1] > 0.1f || it == 6) return RF_SWEEPS;
     rf_gemm<float>(len, vi, n, [&](int k, int i) { return rf_f(__ldcg(m.W + (size_t)k * m.ldw + i)); }, false, F, n, (float*)st, rm,
                    [&](int i, int j, float v) { blk[(size_t)j * len + i] = rf_add(blk[(size_t)j * len + i], v); });
     // V2(:, own) = V(:, own) - V F^T(:, own)
@@ -472,13 +481,12 @@ __device__ __noinline__ bool rf_polish(ClusterCtx& cc, RefineMem<N>& m, int n, i
                      const size_t at = (size_t)(v0 + j) * m.ldv + i;
                      __stcg(m.V2 + at, rf_add(__ldcg(m.V + at), -v));
                    });
-    if (!cl_sync(cc)) return false;                        // W, V and F have been read everywhere
+    if (!cl_sync(cc)) return RF_DEAD;                        // W, V and F have been read everywhere
     { N* t = m.V; m.V = m.V2; m.V2 = t; }
     for (int j = threadIdx.x >> 5; j < vi; j += blockDim.x >> 5)
       for (int k = threadIdx.x & 31; k < len; k += 32) __stcg(m.W + (size_t)(v0 + j) * m.ldw + k, blk[(size_t)j * len + k]);
-    if (!cl_sync(cc)) return false;
+    if (!cl_sync(cc)) return RF_DEAD;
   }
-  return true;
 }
 
 }  // namespace tn

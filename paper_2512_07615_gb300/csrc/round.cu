@@ -843,15 +843,16 @@ __device__ __noinline__ int svd64_rows(ClusterCtx& cc, const RoundJob& J, int L,
     state = rf_refine<N>(cc, rm, ncol, len, sw32 < maxsw, xn, trans, trans, tol2r,
                          two_phase ? 2e-13f : own ? 4e-16f : 1e-16f, own, two_phase ? 2e-6f : 2e-9f, two_phase ? 1e-11f : 1e-14f,
                          two_phase ? 1e-22f : 1e-28f, SM_SMALL, SM_WORK, jacobi);
+    const bool has_w = state == RF_DONE;          // rm.W V^T = X
     tied = rm.tied;
-    if (state == RF_DONE && !trans && !rf_polish<N>(cc, rm, ncol, len, low, tol2r, SM_SMALL, SM_WORK)) state = RF_DEAD;
+    if (state == RF_DONE && !trans) state = rf_polish<N>(cc, rm, ncol, len, low, tol2r, SM_SMALL, SM_WORK);
     if (phase_acc && threadIdx.x == 0) phase_acc[PH_NS] += (double)(clock64() - t0);
     const long long t1 = clock64();
     for (int idx = threadIdx.x; idx < ncol * vi; idx += blockDim.x) {
       const int j = idx / vi, ii = idx % vi;
       Vl[(size_t)j * R.lv + ii] = rf_d(__ldcg(rm.V + (size_t)j * ld1 + v0 + ii));
     }
-    if (state == RF_DONE) {
+    if (has_w) {
       for (int idx = threadIdx.x; idx < ncol * li; idx += blockDim.x) {
         const int j = idx / li, ii = idx % li;
         Wl[(size_t)j * R.lw + ii] = rf_d(__ldcg(rm.W + (size_t)j * rm.ldw + i0 + ii));
