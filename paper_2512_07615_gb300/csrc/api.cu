@@ -843,7 +843,13 @@ template <typename T>
 static int run_round_now(tnlbm_sim* s, std::vector<RoundJob>& jobs) {
   if (jobs.empty()) return 0;
   size_t tot = 0;
-  for (auto& j : jobs) { set_round_options(s, j); plan_round_job(j, s->L, s->n, sizeof(T)); tot += j.lay.total; }
+  const int cl = sim_cluster<T>(s, (int)jobs.size());
+  for (auto& j : jobs) {
+    set_round_options(s, j);
+    if (cl <= 1) j.refine = REFINE_OFF;            // only clusters refine
+    plan_round_job(j, s->L, s->n, sizeof(T));
+    tot += j.lay.total;
+  }
   T* scr = nullptr;
   RoundJob* dj = nullptr;
   if (cudaMalloc(&scr, std::max<size_t>(tot, 1) * sizeof(T)) != cudaSuccess) return TNLBM_E_OOM;
@@ -852,7 +858,7 @@ static int run_round_now(tnlbm_sim* s, std::vector<RoundJob>& jobs) {
   if (cudaMalloc(&dj, jobs.size() * sizeof(RoundJob)) != cudaSuccess) { cudaFree(scr); return TNLBM_E_OOM; }
   cudaMemcpy(dj, jobs.data(), jobs.size() * sizeof(RoundJob), cudaMemcpyHostToDevice);
   launch_round<T>(dj, (int)jobs.size(), s->L, s->n, (const T*)s->d_masks, s->d_scal, s->d_status, s->s0,
-                  nullptr, nullptr, sim_cluster<T>(s, (int)jobs.size()));
+                  nullptr, nullptr, cl);
   cudaError_t e = cudaStreamSynchronize(s->s0);
   cudaFree(scr);
   cudaFree(dj);
@@ -1536,11 +1542,12 @@ static int lincomb_impl(int n_bits, int batch, int nterms, const tnlbm_term* ter
   const int L = 3 * n_bits;
   std::vector<RoundJob> jobs(batch);
   std::vector<T> masks;
+  const int cl = (!materialize && (svd64 || sizeof(T) == 8)) ? round_cluster_size<T>(batch, 16) : 1;
   for (int b = 0; b < batch; ++b) {
     RoundJob& j = jobs[b];
     j = RoundJob{};
     j.svd64 = svd64;
-    j.refine = !materialize && (svd64 || sizeof(T) == 8) ? REFINE_OWN : REFINE_OFF;
+    j.refine = cl > 1 ? REFINE_OWN : REFINE_OFF;   // only clusters refine
     j.nterms = nterms;
     j.chi = chi;
     j.eps = eps;
@@ -1617,7 +1624,6 @@ static int lincomb_impl(int n_bits, int batch, int nterms, const tnlbm_term* ter
   if (!masks.empty()) TN_CUDA(cudaMemcpyAsync(dm.p, masks.data(), masks.size() * sizeof(T), cudaMemcpyHostToDevice, st));
   TN_CUDA(cudaMemsetAsync(ds.p, 0, STATUS_INTS * sizeof(int), st));
   TN_CUDA(cudaMemsetAsync(dsc.p, 0, SC_COUNT * sizeof(double), st));
-  const int cl = (!materialize && (svd64 || sizeof(T) == 8)) ? round_cluster_size<T>(batch, 16) : 1;
   launch_round<T>((const RoundJob*)dj.p, batch, L, n_bits, (const T*)dm.p, (const double*)dsc.p, (int*)ds.p, st,
                   nullptr, ra ? (const LearnCtx*)dlc.p : nullptr, cl);
   TN_CUDA(cudaGetLastError());
