@@ -421,7 +421,9 @@ __device__ __noinline__ int rf_refine(ClusterCtx& cc, RefineMem<N>& m, int n, in
 // sums of 64^3 populations from 1e-14 to 4e-14 off in single cells).  V is then orthonormal to
 // |F| ~ 1e-16 s_0 / s_i only, which its caller multiplies by s_i.  A round squares the sums of
 // a column's cosines and triples them: from 0.1 five rounds end below 1e-16.  Where a sum is
-// larger nothing is done.  low: squared norms (relative to the largest) of columns that are
+// larger nothing is done.  (FP32 data: up to 1.  Such columns are below 1e-9 s_0, all of
+// them rounding, and rarely kept: with 0.1 their sweeps took 10 of 169 ms of a step of 64^3
+// waves.)  low: squared norms (relative to the largest) of columns that are
 // all rounding; they are left out.  RF_DONE; RF_SWEEPS: the sweeps have to finish; or RF_DEAD.
 template <typename N>
 __device__ __noinline__ int rf_polish(ClusterCtx& cc, RefineMem<N>& m, int n, int len, float low, float tol2, int at,
@@ -470,7 +472,7 @@ __device__ __noinline__ int rf_polish(ClusterCtx& cc, RefineMem<N>& m, int n, in
     float s[4] = {rf_block_max(mx, s_red), rf_block_max(sum, s_red), 0.f, 0.f};
     if (!rf_meet_max(cc, m, s)) return RF_DEAD;
     if (s[0] <= tol2) return RF_DONE;
-    if (s[1] > 0.1f || it == 6) return RF_SWEEPS;
+    if (s[1] > (std::is_same<N, double>::value ? 0.1f : 1.f) || it == 6) return RF_SWEEPS;
     rf_gemm<float>(len, vi, n, [&](int k, int i) { return rf_f(__ldcg(m.W + (size_t)k * m.ldw + i)); }, false, F, n, (float*)st, rm,
                    [&](int i, int j, float v) { blk[(size_t)j * len + i] = rf_add(blk[(size_t)j * len + i], v); });
     // V2(:, own) = V(:, own) - V F^T(:, own)
