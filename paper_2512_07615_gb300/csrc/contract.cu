@@ -20,7 +20,10 @@
 //    balanced by powers of two.  The 34 digit products of
 //    weight 256^-7 and more go to eight accumulators in tensor memory, which the epilogue
 //    adds as integers: one rounding per value, four FP64 instructions in place of r.
-//    What is left out is below 2^-59 of the product of the two rows' largest entries.
+//    What is left out, relative to the product of the two rows' largest entries: the products of
+//    weight 256^-8 and less, at most 5 x 128 x 2^-64 and a little, 2^-54.7; and the cut of the
+//    entries to 55 bits, at most 2 x 128 x 2^-56 = 2^-48 (an FP64 sum of 128 rounded products:
+//    2^-46).
 // The digits lie in global memory in the order of the MMA's shared-memory layout
 // (8 x 16-byte core matrices, no swizzle), one bulk copy per operand and K chunk,
 // and the rows of both sides in the order of their coordinates, z fastest, so that a

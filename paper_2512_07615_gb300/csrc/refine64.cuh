@@ -14,7 +14,10 @@
 //
 // The long sums of FP32 data are compensated FP32 sums of exact products on pairs of
 // floats (Ogita, Rump and Oishi's Dot2: 48 bits, 12 instructions a product), as
-// GB300 does 64 FP32 operations in the time of one FP64; FP64 data take FP64.
+// GB300 does 64 FP32 operations in the time of one FP64; FP64 data take FP64.  Against 64-bit
+// results nothing is lost to FP64 sums: kept against discarded directions of 80 matrices of 64 to
+// 180 columns at six and nine decades, rms 1.05e-7 to 2.17e-7 with the pairs, 1.06e-7 to
+// 2.19e-7 with FP64 sweeps in their place (FP32 storage rounds at 6e-8).
 //
 // FP32 sweeps leave the cosine of columns i, j at ~1e-7 s_0 / min(s_i, s_j): nothing
 // for the small ones.  So where a tangent is not small, a second FP32 Jacobi runs on W
@@ -35,8 +38,8 @@
 // goes to the FP64 Jacobi sweeps, started from the V reached.
 //
 // Measured against FP64 sweeps from the V of FP32 sweeps (FP64 data: from V = I): 128^3
-// sums of two at bond 64, mixed, 128 -> 40 ms; 64^3 sums at bond 45, FP64, 83 -> 48 ms; a step
-// of a mixed 64^3 box at bond 32, 342 -> 157 ms.
+// sums of two at bond 64, mixed, 128 -> 40 ms; 64^3 sums at bond 45, FP64, 82 -> 49 ms; a step
+// of a mixed 64^3 box at bond 32, 354 -> 160 ms.
 #pragma once
 
 #include "cluster.cuh"

@@ -1301,8 +1301,8 @@ __device__ __noinline__ int svd32_site(const RoundJob& J, int L, int k, const fl
       }
     }
   }
-  // the padded columns moved among the others: norms of all ncp, the zero ones
-  // (-2) order last and are not counted
+  // the padded columns moved among the others: norms of all ncp; padding is zero like
+  // any column of nothing, and what is not finite orders behind it (and is reported)
   {
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
     for (int j = warp; j < ncp; j += nw) {

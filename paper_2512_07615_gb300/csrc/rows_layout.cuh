@@ -74,8 +74,9 @@ __host__ __device__ inline int rows_stage(int eb, int sw32) {
 // Centre matrices whose sweeps the leader runs alone, as a cluster of one: the exchanges of a
 // round (~3 k of its 9 k cycles) cost more than the other CTAs' FP64 units bring for a
 // few columns, and below ~16 columns the refinement of FP64 data costs more than
-// the sweeps.  Ten channel steps (16^3, FP64): 62.2 -> 56.6 ms on average (58.7 with cluster
-// sweeps throughout), with 12 columns 57.9, 24 as 16, 32 worse for the roundings.  FP32 data
+// the sweeps.  One FP64 step of a 16^3 channel 42.8 -> 36.8 ms, 16^3 wall terms of 18 jobs 7.74 ->
+// 7.04, 32^3 ones 14.5 -> 14.7 (three medians of 15 each, 0.3 % apart).  Ten channel steps with up
+// to 12 columns 57.9 ms, 16 56.6, 24 the same, 32 worse for the roundings.  FP32 data
 // are refined from RF_MIN columns on (16 columns alone: 128^3 sums 55 -> 61 ms).
 static constexpr int SOLO_LEN = 128;
 __host__ __device__ constexpr int solo_cols(int eb) { return eb == 8 ? 16 : RF_MIN - 1; }
